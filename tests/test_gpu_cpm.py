@@ -92,3 +92,32 @@ def test_growth_coupled_to_the_solver(M):
     opts = M.make_opts(rtol=1e-8, restart=16, maxit=500)
     grown, div = _run_pair(M, wl, nc, 6, seed=77, solver_opts=opts)
     assert grown > 0
+
+
+@pytest.mark.parametrize("dims", [(3, 2, 2), (5, 40, 3), (32, 7, 9), (33, 1, 40), (31, 65, 5), (1, 1, 97),
+                                  (200, 43, 2), (96, 64, 8)])
+def test_growth_at_lattice_faces_and_word_edges(M, dims):
+    """Tumour on every face of lattices whose rows are shorter than, equal to
+    and longer than a 32-voxel word, or no multiple of it: bit for bit."""
+    rng = np.random.default_rng(sum(dims))
+    wl, nc = _blob_case(94, dims, ncell=12, cap=60)
+    shape = wl.lattice.cell_id.shape
+    wl.lattice.cell_id = np.where(rng.random(shape) < 0.15, rng.integers(1, nc, size=shape), 0).astype(np.int32)
+    wl.lattice.mask = (rng.random(shape) < 0.9).astype(np.uint8)
+    _run_pair(M, wl, nc, 3, seed=11, cp=dict(CP, p_grow=0.9, v_div=6))
+
+
+def test_ids_outside_the_tables_are_counted_and_left(M):
+    wl, nc = _blob_case(95, (45, 20, 9))
+    wl.lattice.mask[:] = 1
+    c = wl.lattice.cell_id.reshape(-1)
+    c[::37] = -5
+    c[5::41] = 400        # the tables hold 400 entries
+    before = wl.lattice.cell_id.copy()
+    ctx = M.Context()
+    lat, prm = M.DeviceLattice(wl.lattice), M.DeviceParams(wl.params)
+    g = M.GrowthDriver(ctx, lat, prm, nc, seed=3, **dict(CP, p_grow=0.0, v_div=10 ** 6))
+    g.step()
+    assert np.array_equal(lat.cell_id.cpu().numpy(), before)
+    assert g.counts() == {"ncell": nc, "grown": 0, "divisions": 0,
+                          "bad_ids": int(((before < 0) | (before >= 400)).sum())}
