@@ -41,6 +41,10 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
     }
     void *q = nullptr;
     cudaError_t e = cudaMalloc(&q, want);
+    if (e == cudaErrorMemoryAllocation && !ctx->hm_subs.empty()) {   // the face means are optional: give them up
+        while (!ctx->hm_subs.empty()) mpm_face_means_free(ctx, ctx->hm_subs.back());
+        e = cudaMalloc(&q, want);
+    }
     if (e != cudaSuccess) {
         cudaGetLastError();
         return mpm_fail(ctx, MPM_ERR_NOMEM, std::string(what) + ": cudaMalloc of " + std::to_string(want) + " bytes failed");
@@ -51,9 +55,51 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
     return MPM_OK;
 }
 
+// The harmonic means of a per-voxel diffusivity across the faces of n elements:
+// 48 bytes an element, kept between the assembly and the solve so that no pass
+// of the solver divides (an FP64 division costs some ten FP64 instructions, and
+// a pass had six per element).  They are not counted as workspace the caller
+// must provide: a context with a memory cap goes without them, as does one
+// whose device is full, and the solver then forms the means in every pass.
+void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n)
+{
+    if (!sub->has_dfac || ctx->cap || n < 1) {
+        mpm_face_means_free(ctx, sub);
+        return;
+    }
+    const int64_t stride = (n + 31) & ~(int64_t)31;
+    if (6 * stride > sub->hm_cap) {
+        mpm_face_means_free(ctx, sub);
+        const int64_t want = 6 * (stride + stride / 4);
+        double *q = nullptr;
+        if (cudaMalloc(&q, (size_t)want * sizeof(double)) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        sub->hm = q;
+        sub->hm_cap = want;
+        ctx->allocated += (size_t)want * sizeof(double);
+        ctx->hm_subs.push_back(sub);
+    }
+    sub->hm_stride = stride;
+}
+
+void mpm_face_means_free(mpm_ctx *ctx, mpm_subgrid *sub)
+{
+    if (!sub->hm) return;
+    cudaFree(sub->hm);
+    if (ctx) {
+        ctx->allocated -= (size_t)sub->hm_cap * sizeof(double);
+        ctx->hm_subs.erase(std::remove(ctx->hm_subs.begin(), ctx->hm_subs.end(), sub), ctx->hm_subs.end());
+    }
+    sub->hm = nullptr;
+    sub->hm_stride = sub->hm_cap = 0;
+}
+
 static void free_sub_buffers(mpm_ctx *ctx, mpm_subgrid *sub)
 {
     mpm_step_free(ctx, sub);
+    mpm_face_means_free(ctx, sub);
     void **bufs[3] = {&sub->geo, &sub->elem, &sub->krylov};
     size_t *caps[3] = {&sub->geo_bytes, &sub->elem_bytes, &sub->krylov_bytes};
     for (int i = 0; i < 3; ++i) {

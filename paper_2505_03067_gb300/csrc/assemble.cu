@@ -14,6 +14,8 @@ struct AsmArgs {
     const uint8_t *flags;
     const int32_t *cell;
     const double *dfac;
+    double *hm;                 // [6][hstride] or null
+    int64_t hstride;
     const int32_t *tile_coord;
     const int32_t *nbr;
     const double *cn[kMaxSpecies];
@@ -37,6 +39,8 @@ __global__ void __launch_bounds__(kBlock) k_assemble(AsmArgs A, int64_t NE)
                 A.diag32[s][e] = 1.0f;
                 A.b[s][e] = (f & F_BOX) ? A.cn[s][e] : 0.0;
             }
+            if (A.hm)
+                for (int d = 0; d < 6; ++d) A.hm[d * A.hstride + e] = 0.0;
             continue;
         }
         int32_t id = A.cell[e];
@@ -69,9 +73,14 @@ __global__ void __launch_bounds__(kBlock) k_assemble(AsmArgs A, int64_t NE)
             }
             return A.dfac[q];
         };
+        double hm[6], hsum = 0.0;
+        if (A.dfac) hsum = face_means(f, fp, dq, hm);
+        if (A.hm)
+#pragma unroll
+            for (int d = 0; d < 6; ++d) A.hm[d * A.hstride + e] = hm[d];
         for (int s = 0; s < A.C.nspecies; ++s) {
             double dg, b;
-            assemble_row(A.C, s, f, id, ndir, A.dfac != nullptr, fp, dq, A.cn[s][e], dg, b);
+            assemble_row(A.C, s, f, id, ndir, A.dfac != nullptr, fp, hsum, A.cn[s][e], dg, b);
             A.diag[s][e] = dg;
             A.diag32[s][e] = f32_rz(dg);
             A.b[s][e] = b;
@@ -161,6 +170,9 @@ mpm_status mpm_assemble_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_params *p
     A.flags = sub->flags;
     A.cell = sub->cell;
     A.dfac = sub->dfac;
+    mpm_face_means(ctx, sub, sub->NE);
+    A.hm = sub->hm;
+    A.hstride = sub->hm_stride;
     A.tile_coord = sub->tile_coord;
     A.nbr = sub->nbr;
     A.err = sub->err;

@@ -46,6 +46,9 @@ __global__ void k_batch_reset_err(const char *__restrict__ buf, int nsys)
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nsys; i += gridDim.x * blockDim.x) *D[i].err = 0;
 }
 
+// kVar: a system of the batch has a diffusivity factor per voxel.  A batch
+// without one runs a kernel without that code.
+template <bool kVar>
 __global__ void __launch_bounds__(kBlock) k_batch_prep(const char *__restrict__ buf, int nsys)
 {
     const int64_t *blk0 = reinterpret_cast<const int64_t *>(buf);
@@ -54,7 +57,10 @@ __global__ void __launch_bounds__(kBlock) k_batch_prep(const char *__restrict__ 
     const int64_t e0 = (blockIdx.x - blk0[i]) * (int64_t)(kBlock * kEPT);
     const int64_t e1 = min(S.NE, e0 + (int64_t)(kBlock * kEPT));
     const BoxGeo g = S.g;
-    for (int64_t e = e0 + threadIdx.x; e < e1; e += kBlock) prep_elem<false>(S, g, e);
+    for (int64_t e = e0 + threadIdx.x; e < e1; e += kBlock) {
+        if (kVar) prep_elem<false>(S, g, e);
+        else prep_elem_t<false, false>(S, g, e, nullptr, nullptr, nullptr);
+    }
 }
 
 __global__ void __launch_bounds__(kBlock) k_batch_scatter(const char *__restrict__ buf, int nsys)
@@ -129,6 +135,8 @@ mpm_status mpm_batch_desc_fill(mpm_subgrid *const *subs, const mpm_lattice *cons
         S.flags = sub->flags;
         S.cell = sub->cell;
         S.dfac = sub->dfac;
+        S.hm = sub->hm;
+        S.hstride = sub->hm_stride;
         for (int s = 0; s < sub->nspecies; ++s) {
             S.field[s] = lat->field[s];
             S.x[s] = sub->x[s];
@@ -146,12 +154,14 @@ mpm_status mpm_batch_desc_fill(mpm_subgrid *const *subs, const mpm_lattice *cons
     return MPM_OK;
 }
 
-mpm_status mpm_batch_prep_launch(mpm_ctx *ctx, const void *d_desc, int32_t nsys, int64_t nblocks, cudaStream_t st)
+mpm_status mpm_batch_prep_launch(mpm_ctx *ctx, const void *d_desc, int32_t nsys, int64_t nblocks, bool var,
+                                 cudaStream_t st)
 {
     k_batch_reset_err<<<(nsys + kBlock - 1) / kBlock, kBlock, 0, st>>>((const char *)d_desc, nsys);
     ctx->launches += 1;
     if (nblocks > 0) {
-        k_batch_prep<<<(unsigned)nblocks, kBlock, 0, st>>>((const char *)d_desc, nsys);
+        if (var) k_batch_prep<true><<<(unsigned)nblocks, kBlock, 0, st>>>((const char *)d_desc, nsys);
+        else k_batch_prep<false><<<(unsigned)nblocks, kBlock, 0, st>>>((const char *)d_desc, nsys);
         ctx->launches += 1;
     }
     MPM_CU(cudaGetLastError());

@@ -536,6 +536,9 @@ mpm_status mpm_extract_impl(mpm_ctx *ctx, const mpm_lattice *lat, int32_t nspeci
         MPM_CU(cudaGetLastError());
     }
     for (int d = 0; d < 3; ++d) tmp.ldims[d] = lat->dims[d];
+    tmp.hm = sub->hm;   // allocating the buffers above may have given them up
+    tmp.hm_stride = sub->hm_stride;
+    tmp.hm_cap = sub->hm_cap;
     tmp.gen = sub->gen + 1;
     tmp.extracted = true;
     tmp.assembled = false;
@@ -794,6 +797,7 @@ mpm_status mpm_step_buffers(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_lattice *l
     sub->nspecies = nspecies;
     sub->has_dfac = has_dfac;
     sub->NE_cap = (int64_t)NE;
+    mpm_face_means(ctx, sub, (int64_t)NE);
     return MPM_OK;
 }
 

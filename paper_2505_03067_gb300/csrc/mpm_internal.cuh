@@ -150,30 +150,43 @@ struct AsmCoef {
 //   A_PP = 1 + dt (mu_s + k_cell[s][id]) + a (sum_open D_f + 2 D_P n_dir)
 //   b_P  = c^n_P + dt q_cell[s][id] + a 2 D_P c_bc n_dir
 // with D_f the harmonic mean of D_s fp and D_s dq(d) over the open faces d when
-// the diffusivity varies (has_dfac), else D_s on every open face.  n_dir counts
-// the faces of P on the box boundary (Dirichlet c_bc there).  dq(d) returns the
-// diffusivity factor of the neighbour across face d.
-template <typename DQ>
+// the diffusivity varies (has_dfac), else D_s on every open face.  D_s is a
+// factor of every mean, so the means of fp and the neighbours' factors are
+// formed once for all species (face_means: six divisions an element) and hsum
+// is their sum over the open faces.  n_dir counts the faces of P on the box
+// boundary (Dirichlet c_bc there).
 __device__ __forceinline__ void assemble_row(const AsmCoef &C, int s, uint32_t f, int id, int ndir, bool has_dfac,
-                                             double fp, DQ dq, double cn, double &dg, double &b)
+                                             double fp, double hsum, double cn, double &dg, double &b)
 {
     const double kv = C.mu[s] + C.k_cell[(int64_t)s * C.ncell + id];
     if (has_dfac) {
         const double dp = C.D[s] * fp;
-        double acc = 0.0;
-        for (int d = 0; d < 6; ++d) {
-            if (f & (1u << d)) {
-                const double dn = C.D[s] * dq(d);
-                acc += (dp + dn > 0.0) ? 2.0 * dp * dn / (dp + dn) : 0.0;
-            }
-        }
-        dg = 1.0 + C.dt * kv + C.a * (acc + 2.0 * dp * ndir);
+        dg = 1.0 + C.dt * kv + C.a * (C.D[s] * hsum + 2.0 * dp * ndir);
         b = cn + C.dt * C.q_cell[(int64_t)s * C.ncell + id] + C.a * 2.0 * dp * C.cbc[s] * ndir;
     } else {
         const double Ds = C.D[s];
         dg = 1.0 + C.dt * kv + C.a * Ds * (double)(__popc(f & F_OPEN) + 2 * ndir);
         b = cn + C.dt * C.q_cell[(int64_t)s * C.ncell + id] + C.a * 2.0 * Ds * C.cbc[s] * ndir;
     }
+}
+
+// Harmonic means 2 fp fq / (fp + fq) of the diffusivity factors across the six
+// faces (0 on a closed one); dq(d) returns the factor of the neighbour across
+// face d.  Returns their sum.
+template <typename DQ>
+__device__ __forceinline__ double face_means(uint32_t f, double fp, DQ dq, double (&hm)[6])
+{
+    double acc = 0.0;
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+        hm[d] = 0.0;
+        if (f & (1u << d)) {
+            const double fq = dq(d);
+            hm[d] = fp + fq > 0.0 ? 2.0 * fp * fq / (fp + fq) : 0.0;
+            acc += hm[d];
+        }
+    }
+    return acc;
 }
 
 // Device view of one extracted, assembled box system.
@@ -185,6 +198,8 @@ struct SysDev {
     const int32_t *nbr;         // [nact][6] neighbour tile (-1 none): -x,+x,-y,+y,-z,+z
     const uint8_t *flags;       // [NE]
     const double *dfac;         // [NE] or null (uniform D)
+    const double *hm;           // [6][hstride] harmonic means of dfac across the faces, or null
+    int64_t hstride;
     double *x[kMaxSpecies];     // iterate (FP64)
     const double *b[kMaxSpecies];
     const double *diag[kMaxSpecies];
@@ -440,6 +455,7 @@ struct mpm_ctx {
     std::vector<double> item_cta;       //   CTAs of its team
     std::vector<double> item_ns;        //   device time (its team's CTA 0)
     std::vector<double> team_ns;        // per team of the last solve: device time
+    std::vector<mpm_subgrid *> hm_subs;   // subgrids holding face means (given up when memory runs out)
     int64_t step_nfull = 0;      // mpm_step: full extractions so far (MPM_COUNTER_STEP_FULL_EXTRACTIONS)
     // test hooks
     uint64_t timeout_ns = 2000000000ull;
@@ -474,6 +490,11 @@ struct mpm_subgrid {
     uint8_t *flags = nullptr;
     int32_t *cell = nullptr;
     double *dfac = nullptr;
+    // harmonic means of dfac across the six faces, [6][hm_stride], written by the
+    // assembly and read by the solver; optional (mpm_face_means): without it the
+    // solver forms them in every pass
+    double *hm = nullptr;
+    int64_t hm_stride = 0, hm_cap = 0;   // doubles per face, doubles allocated
     double *x[MPM_MAX_SPECIES] = {};
     double *cn[MPM_MAX_SPECIES] = {};
     double *b[MPM_MAX_SPECIES] = {};
@@ -492,6 +513,8 @@ struct mpm_subgrid {
 mpm_status mpm_fail(mpm_ctx *ctx, mpm_status st, const std::string &msg);
 mpm_status mpm_cuda_check(mpm_ctx *ctx, cudaError_t e, const char *what);
 mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char *what);
+void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n);   // room for the face means of n elements, if any
+void mpm_face_means_free(mpm_ctx *ctx, mpm_subgrid *sub);
 
 #define MPM_CU(call)                                                       \
     do {                                                                   \
@@ -518,7 +541,8 @@ mpm_status mpm_batch_prep_check(mpm_ctx *ctx, mpm_subgrid *const *subs, const mp
                                 const mpm_params *const *prms, int32_t nsys);
 mpm_status mpm_batch_desc_fill(mpm_subgrid *const *subs, const mpm_lattice *const *lats,
                                const mpm_params *const *prms, int32_t nsys, void *host, int64_t *nblocks);
-mpm_status mpm_batch_prep_launch(mpm_ctx *ctx, const void *d_desc, int32_t nsys, int64_t nblocks, cudaStream_t st);
+mpm_status mpm_batch_prep_launch(mpm_ctx *ctx, const void *d_desc, int32_t nsys, int64_t nblocks, bool var,
+                                 cudaStream_t st);
 mpm_status mpm_batch_scatter_launch(mpm_ctx *ctx, const void *d_desc, int32_t nsys, int64_t nblocks, cudaStream_t st);
 // extraction with buffers sized for the whole lattice and no host round trip (extract.cu)
 mpm_status mpm_step_buffers(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_lattice *lat, int32_t nspecies, const int32_t lt[3]);

@@ -20,8 +20,12 @@ namespace mpm {
 // element at one CTA/SM of 1024, 3: one element at one CTA/SM of 768, 4: two
 // elements at one CTA/SM of 768, 5: one element at one CTA/SM of 512.
 // The instances live in the solver_inst_*.cu translation units.
-static Variant pick(int prec, int maxm, int variant)
+static Variant pick(int prec, int maxm, int variant, bool var)
 {
+    if (var) {   // a per-voxel diffusivity: the default of each bucket only
+        if (prec != 0) return maxm == 8 ? inst_f32_8_var() : maxm == 16 ? inst_f32_16_var() : inst_f32_32_var();
+        return maxm == 8 ? inst_f64_8_var() : maxm == 16 ? inst_f64_16_var() : inst_f64_32_var();
+    }
     if (prec != 0) {
         if (maxm == 16) return inst_f32_16_1_1_512();
         if (maxm == 32) return inst_f32_32_1_1_512();
@@ -63,6 +67,8 @@ SysDev mpm_make_sysdev(const mpm_subgrid *sub)
     S.nbr = sub->nbr;
     S.flags = sub->flags;
     S.dfac = sub->dfac;
+    S.hm = sub->hm;
+    S.hstride = sub->hm_stride;
     S.a = sub->a;
     S.err = sub->err;
     for (int s = 0; s < sub->nspecies; ++s) {
@@ -86,10 +92,10 @@ static int variant_max_blocks(mpm_ctx *ctx, const Variant &v, bool step)
     return per_sm * ctx->num_sms;
 }
 
-int mpm_solver_max_blocks(mpm_ctx *ctx, int prec, int m, int variant)
+int mpm_solver_max_blocks(mpm_ctx *ctx, int prec, int m, int variant, bool var)
 {
     const int maxm = m <= 8 ? 8 : (m <= 16 ? 16 : 32);
-    return variant_max_blocks(ctx, pick(prec, maxm, variant), false);
+    return variant_max_blocks(ctx, pick(prec, maxm, variant, var), false);
 }
 
 // Number of kernel variants of a (precision, restart) bucket (for the tuner).
@@ -271,8 +277,10 @@ static mpm_status plan_solve(mpm_ctx *ctx, mpm_subgrid *const *subs, int nsys, c
         if (!subs[i]->assembled && reset_x) return mpm_fail(ctx, MPM_ERR_ARG, "solve: subgrid not assembled");
     }
     std::vector<double> work;
+    bool any_var = false;   // a system with a per-voxel diffusivity
     for (int i = 0; i < nsys; ++i) {
         mpm_subgrid *sub = subs[i];
+        any_var |= sub->has_dfac;
         const int64_t ne_v = ov ? ov->NE_cap : sub->NE;
         const int64_t vstride = ne_v > 0 ? ((ne_v + 63) / 64) * 64 : 64;
         const size_t per = a256((size_t)(m + 1) * (size_t)vstride * tsz);
@@ -311,13 +319,13 @@ static mpm_status plan_solve(mpm_ctx *ctx, mpm_subgrid *const *subs, int nsys, c
     }
     P.nitem = (int)P.sd.size();
     {
-        const Variant v = pick(opt->precision, maxm, ctx->solver_variant);
+        const Variant v = pick(opt->precision, maxm, ctx->solver_variant, any_var);
         P.fn = v.fn;
         P.stepfn = v.stepfn;
         P.smem = v.smem;
         P.nt = v.nt;
     }
-    const int gmax = mpm_solver_max_blocks(ctx, opt->precision, m, ctx->solver_variant);
+    const int gmax = mpm_solver_max_blocks(ctx, opt->precision, m, ctx->solver_variant, any_var);
     if (gmax < 1) return mpm_fail(ctx, MPM_ERR_CUDA, "solve: occupancy query failed");
     if (ov && ov->G > 0) P.G = std::min(ov->G, gmax);
     else if (opt->nblocks > 0) P.G = std::min(opt->nblocks, gmax);
@@ -380,8 +388,14 @@ static mpm_status plan_solve(mpm_ctx *ctx, mpm_subgrid *const *subs, int nsys, c
     return MPM_OK;
 }
 
-static void fill_descriptors(const SolvePlan &P, char *h)
+// subs: the plan's subgrids.  Their face means are looked up here, after the
+// last allocation of the call (an allocation may give them up).
+static void fill_descriptors(SolvePlan &P, mpm_subgrid *const *subs, char *h)
 {
+    for (int i = 0; i < P.nitem; ++i) {
+        P.sd[i].hm = subs[P.item_sys[i]]->hm;
+        P.sd[i].hstride = subs[P.item_sys[i]]->hm_stride;
+    }
     memcpy(h + P.o_sys, P.sd.data(), sizeof(SysDev) * P.nitem);
     memcpy(h + P.o_team, P.teams.data(), sizeof(TeamDesc) * P.nteam);
     memcpy(h + P.o_order, P.order.data(), sizeof(int32_t) * P.nitem);
@@ -530,7 +544,7 @@ mpm_status mpm_solve_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm_latt
     if (ctx->phase_prof && !ctx->d_prof) MPM_CU(cudaMalloc(&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
     // the staging buffer is free: every call that uses it ends with a stream synchronisation
     char *hs = (char *)ctx->h_stage;
-    fill_descriptors(P, hs);
+    fill_descriptors(P, subs, hs);
     MPM_CU(cudaMemcpyAsync(ctx->d_args, hs, P.o_rep, cudaMemcpyHostToDevice, st));
     MPM_CU(cudaEventRecord(ctx->ev0, st));
     r = enqueue_solve(ctx, P, (char *)ctx->d_args, ctx->d_bar, ctx->d_abort, ctx->phase_prof ? ctx->d_prof : nullptr, st);
@@ -587,6 +601,8 @@ static void batch_key(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm_lattice 
         put(&subs[i], sizeof(void *));
         put(&subs[i]->gen, sizeof(subs[i]->gen));
         put(&subs[i]->krylov, sizeof(void *));
+        put(&subs[i]->hm, sizeof(void *));
+        put(&subs[i]->hm_stride, sizeof(int64_t));
         put(lats[i], sizeof(mpm_lattice));
         put(prms[i], sizeof(mpm_params));
     }
@@ -620,6 +636,11 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
     if (r != MPM_OK) return r;
     if (!ctx->batch_graph) ctx->batch_graph = new BatchGraph();
     BatchGraph *B = (BatchGraph *)ctx->batch_graph;
+    bool var = false;   // part of the key: gen changes with the extraction, and dfac's presence with it
+    for (int i = 0; i < nsys; ++i) {
+        mpm_face_means(ctx, subs[i], subs[i]->NE);
+        var |= subs[i]->has_dfac;
+    }
     std::vector<unsigned char> key;
     batch_key(ctx, subs, lats, prms, nsys, opt, key);
     const bool use_graph = !ctx->phase_prof;
@@ -634,7 +655,7 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
         r = mpm_grow(ctx, (void **)&B->d_desc, &B->desc_cap, dbytes, "batch preparation descriptors");
         if (r != MPM_OK) return r;
         MPM_CU(cudaMemcpyAsync(B->d_desc, B->h_desc.data(), dbytes, cudaMemcpyHostToDevice, st));
-        r = mpm_batch_prep_launch(ctx, B->d_desc, nsys, B->prep_blocks, st);
+        r = mpm_batch_prep_launch(ctx, B->d_desc, nsys, B->prep_blocks, var, st);
         if (r != MPM_OK) return r;
         for (int i = 0; i < nsys; ++i) { subs[i]->assembled = true; subs[i]->x_fresh = true; }
         B->plan = SolvePlan();
@@ -653,7 +674,10 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
         if (B->plan.nteam > ctx->num_sms * 4) return mpm_fail(ctx, MPM_ERR_ARG, "batch_step: too many teams");
         r = ensure_stage(ctx, B->plan.args_need + 4096);
         if (r != MPM_OK) return r;
-        fill_descriptors(B->plan, (char *)ctx->h_stage);
+        fill_descriptors(B->plan, subs, (char *)ctx->h_stage);
+        // the preparation's descriptors as well (same reason)
+        mpm_batch_desc_fill(subs, lats, prms, nsys, B->h_desc.data(), &B->prep_blocks);
+        MPM_CU(cudaMemcpyAsync(B->d_desc, B->h_desc.data(), dbytes, cudaMemcpyHostToDevice, st));
         MPM_CU(cudaMemcpyAsync(B->d_args, ctx->h_stage, B->plan.o_rep, cudaMemcpyHostToDevice, st));
         MPM_CU(cudaStreamSynchronize(st));   // descriptors in place before any capture
         if (use_graph && !B->graph_failed) {
@@ -666,7 +690,7 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
             const int64_t launches0 = ctx->launches;
             bool ok = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
             if (ok) {
-                ok = mpm_batch_prep_launch(ctx, B->d_desc, nsys, B->prep_blocks, cs) == MPM_OK;
+                ok = mpm_batch_prep_launch(ctx, B->d_desc, nsys, B->prep_blocks, var, cs) == MPM_OK;
                 ok = ok && enqueue_solve(ctx, B->plan, B->d_args, B->d_bar, B->d_abort, nullptr, cs) == MPM_OK;
                 ok = ok && mpm_batch_scatter_launch(ctx, B->d_desc, nsys, B->prep_blocks, cs) == MPM_OK;
                 const cudaError_t ec = cudaStreamEndCapture(cs, &g);
@@ -696,7 +720,7 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
         ctx->launches += B->graph_launches;
     } else {
         // eager form of the same sequence (graph unavailable or phase timing on)
-        r = mpm_batch_prep_launch(ctx, B->d_desc, nsys, B->prep_blocks, st);
+        r = mpm_batch_prep_launch(ctx, B->d_desc, nsys, B->prep_blocks, var, st);
         if (r != MPM_OK) return r;
         if (ctx->phase_prof && !ctx->d_prof) MPM_CU(cudaMalloc(&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
         r = enqueue_solve(ctx, P, B->d_args, B->d_bar, B->d_abort, ctx->phase_prof ? ctx->d_prof : nullptr, st);
@@ -754,7 +778,7 @@ struct StepGraph {
     // what mpm_step_wait needs from the last enqueued step
     bool pending = false;
     int32_t margin = 0, lt[3] = {2, 2, 2}, ldims[3] = {0, 0, 0};
-    int gmax_key[3] = {-1, -1, -1};  // (precision, restart bucket, variant) of the cached grid limit
+    int gmax_key[4] = {-1, -1, -1, -1};  // (precision, restart bucket, variant, dfac) of the cached grid limit
     int gmax = 0;
     mpm_cnn *cnn = nullptr;          // the network whose prediction starts each solve (null: c^n)
 };
@@ -804,6 +828,8 @@ static BatchSys step_sys(mpm_subgrid *sub, const mpm_lattice *lat, const mpm_par
     S.flags = sub->flags;
     S.cell = sub->cell;
     S.dfac = sub->dfac;
+    S.hm = sub->hm;
+    S.hstride = sub->hm_stride;
     for (int s = 0; s < sub->nspecies; ++s) {
         S.field[s] = lat->field[s];
         S.x[s] = sub->x[s];
@@ -952,12 +978,15 @@ mpm_status mpm_step_enqueue_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_latti
     // grid: from the previous step's element count, kept while within 25%;
     // at most the co-resident CTAs of the whole-step kernel
     const int maxm = opt->restart <= 8 ? 8 : (opt->restart <= 16 ? 16 : 32);
-    const Variant var = pick(opt->precision, maxm, ctx->solver_variant);
-    if (T->gmax_key[0] != opt->precision || T->gmax_key[1] != maxm || T->gmax_key[2] != ctx->solver_variant) {
+    const int has_dfac = lat->dfac != nullptr;
+    const Variant var = pick(opt->precision, maxm, ctx->solver_variant, has_dfac);
+    if (T->gmax_key[0] != opt->precision || T->gmax_key[1] != maxm || T->gmax_key[2] != ctx->solver_variant ||
+        T->gmax_key[3] != has_dfac) {
         T->gmax = variant_max_blocks(ctx, var, true);   // occupancy query: once per variant
         T->gmax_key[0] = opt->precision;
         T->gmax_key[1] = maxm;
         T->gmax_key[2] = ctx->solver_variant;
+        T->gmax_key[3] = has_dfac;
     }
     const int gmax = T->gmax;
     if (gmax < 1) return mpm_fail(ctx, MPM_ERR_CUDA, "step: occupancy query failed");
@@ -988,6 +1017,8 @@ mpm_status mpm_step_enqueue_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_latti
         put(&sub->geo, sizeof(void *));
         put(&sub->elem, sizeof(void *));
         put(&sub->krylov, sizeof(void *));
+        put(&sub->hm, sizeof(void *));
+        put(&sub->hm_stride, sizeof(int64_t));
         put(&T->cnn, sizeof(void *));
     };
     std::vector<unsigned char> key;
@@ -1032,7 +1063,8 @@ mpm_status mpm_step_enqueue_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_latti
         if (ctx->phase_prof && !ctx->d_prof) MPM_CU(cudaMalloc(&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
         r = ensure_stage(ctx, T->plan.args_need + 4096);
         if (r != MPM_OK) return r;
-        fill_descriptors(T->plan, (char *)ctx->h_stage);
+        fill_descriptors(T->plan, &sub, (char *)ctx->h_stage);
+        make_key(key);   // the allocations may have given up the face means
         MPM_CU(cudaMemcpyAsync(T->d_args, ctx->h_stage, T->plan.o_rep, cudaMemcpyHostToDevice, st));
         // between-step state at its initial values: activity bytes, grid barrier
         // and exit counters, team barrier counters and the abort flag at zero

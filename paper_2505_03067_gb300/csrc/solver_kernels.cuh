@@ -1,7 +1,7 @@
 // solver_kernels.cuh -- restarted GMRES (Saad & Schultz 1986, the solver named
 // in Sec. 2.4) for the box systems, as ONE persistent cooperative kernel: the
 // device code and its instantiation helper (the instances themselves live
-// in the solver_inst_*.cu translation units, two each, compiled in
+// in the solver_inst_*.cu translation units, two each at most, compiled in
 // parallel).
 //
 // Structure of a launch.  The grid is split into teams of co-resident CTAs;
@@ -231,6 +231,47 @@ __device__ __forceinline__ T open_sum_var(const T *__restrict__ u, const double 
     return s;
 }
 
+// The FP32 value of a positive normal-range x (or zero) rounded to nearest even by
+// integer operations, as f32_rz for the conversions off the FP64 pipe; other
+// values as f32_rz gives them.
+__device__ __forceinline__ float f32_rn(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    return f32_rz(__longlong_as_double((long long)(b + 0x0fffffffull + ((b >> 29) & 1ull))));
+}
+__device__ __forceinline__ double mean_as(double x, double) { return x; }
+__device__ __forceinline__ float mean_as(double x, float) { return f32_rn(x); }
+
+// The same with the means of the diffusivity factors stored by the assembly
+// (D_s, and dt / h^2, left to the caller): six multiply-adds and no division.
+// A closed face has mean 0 and reads e itself.
+template <typename T>
+__device__ __forceinline__ T open_sum_hm(const T *__restrict__ u, const double *__restrict__ hm, int64_t hs, uint32_t e,
+                                         const uint32_t (&q)[6])
+{
+    T v[6];
+    double h[6];
+#pragma unroll
+    for (int d = 0; d < 6; ++d) {
+        v[d] = __ldcg(u + q[d]);
+        h[d] = ldro(hm + d * hs + e);
+    }
+    T a = mean_as(h[0], T(0)) * v[0], b = mean_as(h[1], T(0)) * v[1];
+    a += mean_as(h[2], T(0)) * v[2];
+    b += mean_as(h[3], T(0)) * v[3];
+    a += mean_as(h[4], T(0)) * v[4];
+    b += mean_as(h[5], T(0)) * v[5];
+    return a + b;
+}
+
+// Forms of the stencil's coefficients: D_s on every open face, harmonic means
+// of a per-voxel factor formed in the pass, or stored ones.  Stored means take
+// 48 bytes an element; the other form is for a subgrid without them.  On a
+// 97x150x121 lattice with four species in FP64 (193 k unknowns) extraction,
+// assembly, solve and scatter took 1570 us with the means formed in every pass
+// (solve 1175, assembly 193) and take 632 us with stored ones.
+enum { D_UNIFORM = 0, D_MEANS = 1, D_STORED = 2 };
+
 // Every pass handles U elements per thread and iteration (e, e+es, ...,
 // spaced one grid stride apart) and issues all their loads before the first
 // store: stores through the Krylov base pointer may alias later loads in the
@@ -246,7 +287,7 @@ __device__ __forceinline__ double to_basis<double>(double x) { return x; }
 
 // ---- R: r = b - A x in FP64; u_0 = r (stored in T); sums of r^2 and of b^2
 // over mask rows.
-template <typename T, int U, bool VAR>
+template <typename T, int U, int VAR>
 __device__ __forceinline__ void pass_residual_t(const SysDev &S, bool first, uint32_t e0, uint32_t es,
                                                 double &aR, double &aB)
 {
@@ -254,7 +295,7 @@ __device__ __forceinline__ void pass_residual_t(const SysDev &S, bool first, uin
     // values would underflow for fields below ~1e-19 and end the solve on a
     // zero norm.
     const uint32_t NE = (uint32_t)S.NE;
-    constexpr bool var = VAR;
+    constexpr bool var = VAR == D_MEANS;
     const double *x = S.x[0];
     // the flag bytes and the tile's neighbour entries are read-only during the
     // solve: fetch the next iteration's one iteration ahead, so the neighbour
@@ -285,7 +326,9 @@ __device__ __forceinline__ void pass_residual_t(const SysDev &S, bool first, uin
             const uint32_t eu = e + u * es;
             if (eu >= NE) continue;
             xv[u] = __ldcg(x + eu);   // the update may have written it from another CTA
-            ns[u] = var ? S.a * open_sum_var<double>(x, S.dfac, eu, f[u], q[u], S.Dsp[0]) : open_sum_sel<double>(x, f[u], q[u]);
+            if (var) ns[u] = S.a * open_sum_var<double>(x, S.dfac, eu, f[u], q[u], S.Dsp[0]);
+            else if (VAR == D_STORED) ns[u] = open_sum_hm<double>(x, S.hm, S.hstride, eu, q[u]);
+            else ns[u] = open_sum_sel<double>(x, f[u], q[u]);
             bv[u] = ldro(S.b[0] + eu);
             dg[u] = ldro(S.diag[0] + eu);
         }
@@ -302,24 +345,25 @@ __device__ __forceinline__ void pass_residual_t(const SysDev &S, bool first, uin
     }
 }
 
-// the harmonic-mean (per-voxel D) and the uniform-D form as separate loops
-template <typename T, int U>
+// VAR: the kernel may meet systems with a per-voxel diffusivity.
+template <typename T, int U, bool VAR>
 __device__ __forceinline__ void pass_residual(const SysDev &S, bool first, uint32_t e0, uint32_t es,
                                               double &aR, double &aB)
 {
-    if (S.dfac) pass_residual_t<T, U, true>(S, first, e0, es, aR, aB);
-    else pass_residual_t<T, U, false>(S, first, e0, es, aR, aB);
+    if (VAR && S.hm) pass_residual_t<T, U, D_STORED>(S, first, e0, es, aR, aB);
+    else if (VAR && S.dfac) pass_residual_t<T, U, D_MEANS>(S, first, e0, es, aR, aB);
+    else pass_residual_t<T, U, D_UNIFORM>(S, first, e0, es, aR, aB);
 }
 
 // ---- P1: w = sigma_j A u_j into slot j+1; acc[i] += u_i . w for i <= j
-template <typename T, int MAXM, int U, bool VAR, int JJ = -1, int LIM = MAXM>
+template <typename T, int MAXM, int U, int VAR, int JJ = -1, int LIM = MAXM>
 __device__ __forceinline__ void pass_arnoldi1_t(const SysDev &S, int jr, T sj, uint32_t e0, uint32_t es,
                                                 T (&acc)[MAXM + 1], bool want_ww)
 {
     const int j = JJ >= 0 ? JJ : jr;   // JJ >= 0: the step index known at compile time
     const uint32_t NE = (uint32_t)S.NE;
     const int64_t vs = S.vstride;
-    constexpr bool var = VAR;
+    constexpr bool var = VAR == D_MEANS;
     const T offT = (T)(var ? S.a : S.off[0]);
     const T *V = (const T *)S.V[0];
     const T *uj = V + (int64_t)j * vs;
@@ -352,7 +396,9 @@ __device__ __forceinline__ void pass_arnoldi1_t(const SysDev &S, int jr, T sj, u
             const uint32_t eu = e + u * es;
             if (eu >= NE) continue;
             xj[u] = __ldcg(uj + eu);   // the chunked passes may have written these from other CTAs
-            ns[u] = var ? open_sum_var<T>(uj, S.dfac, eu, f[u], q[u], S.Dsp[0]) : open_sum<T>(uj, f[u], q[u]);
+            if (var) ns[u] = open_sum_var<T>(uj, S.dfac, eu, f[u], q[u], S.Dsp[0]);
+            else if (VAR == D_STORED) ns[u] = open_sum_hm<T>(uj, S.hm, S.hstride, eu, q[u]);
+            else ns[u] = open_sum<T>(uj, f[u], q[u]);
             dg[u] = ldro(dgp + eu);
 #pragma unroll
             for (int i = 0; i < LIM; ++i) vi[u][i] = i < j ? __ldcg(V + (int64_t)i * vs + eu) : T(0);
@@ -528,23 +574,27 @@ __device__ __forceinline__ void pass_arnoldi1_rows(const SysDev &S, int j, T sj,
     }
 }
 
-template <typename T, int MAXM, int U>
+template <typename T, int MAXM, int U, int FORM>
+__device__ __forceinline__ void pass_arnoldi1_form(const SysDev &S, int j, T sj, uint32_t e0, uint32_t es,
+                                                   T (&acc)[MAXM + 1], bool want_ww)
+{
+    if (exact_j<T, MAXM>())
+        with_exact(j, [&](auto J) { pass_arnoldi1_t<T, MAXM, U, FORM, decltype(J)::value>(S, j, sj, e0, es, acc, want_ww); });
+    else
+        with_limit<MAXM>(j, [&](auto L) {
+            constexpr int LIM = decltype(L)::value;
+            if (FORM == D_UNIFORM && use_rows<T>(S)) pass_arnoldi1_rows<T, MAXM, LIM>(S, j, sj, e0, es, acc, want_ww);
+            else pass_arnoldi1_t<T, MAXM, U, FORM, -1, LIM>(S, j, sj, e0, es, acc, want_ww);
+        });
+}
+
+template <typename T, int MAXM, int U, bool VAR>
 __device__ __forceinline__ void pass_arnoldi1(const SysDev &S, int j, T sj, uint32_t e0, uint32_t es,
                                               T (&acc)[MAXM + 1], bool want_ww)
 {
-    if (exact_j<T, MAXM>()) {
-        if (S.dfac)
-            with_exact(j, [&](auto J) { pass_arnoldi1_t<T, MAXM, U, true, decltype(J)::value>(S, j, sj, e0, es, acc, want_ww); });
-        else
-            with_exact(j, [&](auto J) { pass_arnoldi1_t<T, MAXM, U, false, decltype(J)::value>(S, j, sj, e0, es, acc, want_ww); });
-    } else {
-        with_limit<MAXM>(j, [&](auto L) {
-            constexpr int LIM = decltype(L)::value;
-            if (S.dfac) pass_arnoldi1_t<T, MAXM, U, true, -1, LIM>(S, j, sj, e0, es, acc, want_ww);
-            else if (use_rows<T>(S)) pass_arnoldi1_rows<T, MAXM, LIM>(S, j, sj, e0, es, acc, want_ww);
-            else pass_arnoldi1_t<T, MAXM, U, false, -1, LIM>(S, j, sj, e0, es, acc, want_ww);
-        });
-    }
+    if (VAR && S.hm) pass_arnoldi1_form<T, MAXM, U, D_STORED>(S, j, sj, e0, es, acc, want_ww);
+    else if (VAR && S.dfac) pass_arnoldi1_form<T, MAXM, U, D_MEANS>(S, j, sj, e0, es, acc, want_ww);
+    else pass_arnoldi1_form<T, MAXM, U, D_UNIFORM>(S, j, sj, e0, es, acc, want_ww);
 }
 
 // ---- P2: w -= sum_{i<=j} c_i u_i in place (c_i = h_ij sigma_i); acc += w^2
@@ -735,7 +785,7 @@ __device__ __forceinline__ void pass_update(const SysDev &S, int k, const T *c, 
 
 // The persistent GMRES of one CTA of a team (every item of its team in turn).
 // Returns early when a team barrier gave up (the abort flag is then set).
-template <typename T, int MAXM, int U, int NT>
+template <typename T, int MAXM, int U, int NT, bool VAR>
 __device__ __forceinline__ void gmres_body(const SolveArgs &A, Smem<MAXM, T, NT> &sm)
 {
     const int tid = threadIdx.x;
@@ -799,7 +849,7 @@ __device__ __forceinline__ void gmres_body(const SolveArgs &A, Smem<MAXM, T, NT>
             wcat = 4;
             if (rmask & 1u) {
                 double a2[1][2] = {{0.0, 0.0}};
-                pass_residual<T, U>(S, first, e0, es, a2[0][0], a2[0][1]);
+                pass_residual<T, U, VAR>(S, first, e0, es, a2[0][0], a2[0][1]);
                 block_reduce_g<1, 2, double, NT>(a2, 1u, 2, 0, sm.red, mypart);
             }
             MPM_BARRIER();
@@ -845,7 +895,7 @@ __device__ __forceinline__ void gmres_body(const SolveArgs &A, Smem<MAXM, T, NT>
                     T acc[1][MAXM + 1];
 #pragma unroll
                     for (int i = 0; i <= MAXM; ++i) acc[0][i] = T(0);
-                    pass_arnoldi1<T, MAXM, U>(S, j, sm.sig[0][j], e0, es, acc[0], A.reorth != 0);
+                    pass_arnoldi1<T, MAXM, U, VAR>(S, j, sm.sig[0][j], e0, es, acc[0], A.reorth != 0);
                     block_reduce_g<1, MAXM + 1, T, NT>(acc, 1u, j + 1 + (A.reorth != 0), 0, sm.red, mypart);
                 }
                 MPM_BARRIER();
@@ -1022,13 +1072,17 @@ __device__ __forceinline__ void gmres_body(const SolveArgs &A, Smem<MAXM, T, NT>
 
 // U: elements in flight per thread in the streaming passes; MINB: CTAs per SM
 // the register allocation must allow (1: up to 128 registers, 2: up to 64).
-template <typename T, int MAXM, int U, int MINB, int NT>
+// VAR: some system of the launch has a per-voxel diffusivity.  Launches
+// without one run kernels without that code: beside it, inlined or not, the
+// uniform passes lost 2-3 % (256^3 shell 237 -> 244 us a step) to register
+// pressure.
+template <typename T, int MAXM, int U, int MINB, int NT, bool VAR>
 __global__ void __launch_bounds__(NT, MINB) k_gmres(SolveArgs A)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
     Smem<MAXM, T, NT> &sm = *reinterpret_cast<Smem<MAXM, T, NT> *>(smraw);
     if ((int)blockIdx.x == A.skip_block) return;    // fault injection: this CTA never arrives
-    gmres_body<T, MAXM, U, NT>(A, sm);
+    gmres_body<T, MAXM, U, NT, VAR>(A, sm);
 }
 
 // ------------------------------------------------------------------ the whole step in one kernel
@@ -1063,7 +1117,7 @@ struct StepArgs {
 // grid barrier, the scatter onto the pleural mask (skipped if any wait gave
 // up).  The last CTA to leave copies the results to host-mapped memory and
 // resets the grid barrier and exit counters for the next step.
-template <typename T, int MAXM, int U, int MINB, int NT>
+template <typename T, int MAXM, int U, int MINB, int NT, bool VAR>
 __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepArgs P)
 {
     extern __shared__ __align__(16) unsigned char smraw[];
@@ -1079,14 +1133,14 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
     if (b != P.sa.skip_block && P.mode == STEP_EXTRACT) {
         // the extraction alone; the kernel boundary orders it before the guess
         uint32_t epoch = 0;
-        if (full) extract_phases<NT>(P.xa, P.S, b, nb, epoch);
-        else refresh_phases<NT>(P.xa, P.S, b, nb, epoch);
+        if (full) extract_phases<NT, VAR>(P.xa, P.S, b, nb, epoch);
+        else refresh_phases<NT, VAR>(P.xa, P.S, b, nb, epoch);
         if (prof) P.sa.prof[8] += globaltimer_ns() - t0;
     } else if (b != P.sa.skip_block) {              // fault injection: this CTA never arrives
         uint32_t epoch = 0;
         bool ok = true;
         if (P.mode == STEP_WHOLE) {
-            ok = full ? extract_phases<NT>(P.xa, P.S, b, nb, epoch) : refresh_phases<NT>(P.xa, P.S, b, nb, epoch);
+            ok = full ? extract_phases<NT, VAR>(P.xa, P.S, b, nb, epoch) : refresh_phases<NT, VAR>(P.xa, P.S, b, nb, epoch);
             ok = ok && team_barrier(P.xa.bar, epoch, nb, P.xa.xabort, P.xa.timeout_ns);
         } else {
             ok = *(volatile int32_t *)P.xa.xabort == 0;   // the extraction launch gave up
@@ -1095,7 +1149,7 @@ __global__ void __launch_bounds__(NT, MINB) k_step(const __grid_constant__ StepA
             const uint64_t t = globaltimer_ns();
             P.sa.prof[8] += t - t0;
         }
-        if (ok) gmres_body<T, MAXM, U, NT>(P.sa, sm);
+        if (ok) gmres_body<T, MAXM, U, NT, VAR>(P.sa, sm);
         if (prof) t0 = globaltimer_ns();
         ok = ok && team_barrier(P.xa.bar, epoch, nb, P.xa.xabort, P.xa.timeout_ns);
         if (ok && *(volatile int32_t *)P.xa.xabort == 0) {
@@ -1165,14 +1219,14 @@ struct Variant {
     int nt;
 };
 
-template <typename T, int MAXM, int U, int MINB, int NT>
+template <typename T, int MAXM, int U, int MINB, int NT, bool VAR = false>
 static Variant var_of()
 {
-    return Variant{k_gmres<T, MAXM, U, MINB, NT>, k_step<T, MAXM, U, MINB, NT>, sizeof(Smem<MAXM, T, NT>), NT};
+    return Variant{k_gmres<T, MAXM, U, MINB, NT, VAR>, k_step<T, MAXM, U, MINB, NT, VAR>, sizeof(Smem<MAXM, T, NT>), NT};
 }
 
 // Kernel instances <type, restart bucket, elements per thread, CTAs per SM,
-// threads>, defined in the solver_inst_*.cu translation units.
+// threads> (uniform diffusivity), defined in the solver_inst_*.cu translation units.
 Variant inst_f32_8_1_1_512();
 Variant inst_f32_8_1_1_768();
 Variant inst_f32_8_2_2_512();
@@ -1190,5 +1244,12 @@ Variant inst_f64_8_1_1_768();
 Variant inst_f64_8_2_1_768();
 Variant inst_f64_16_1_1_512();
 Variant inst_f64_32_1_1_512();
+// with a per-voxel diffusivity: one instance per precision and restart bucket
+Variant inst_f32_8_var();
+Variant inst_f32_16_var();
+Variant inst_f32_32_var();
+Variant inst_f64_8_var();
+Variant inst_f64_16_var();
+Variant inst_f64_32_var();
 
 }  // namespace mpm

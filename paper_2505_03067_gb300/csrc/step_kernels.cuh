@@ -21,6 +21,8 @@ struct BatchSys {
     uint8_t *flags;
     int32_t *cell;
     double *dfac;
+    double *hm;                 // [6][hstride] face means of dfac, or null
+    int64_t hstride;
     double *x[kMaxSpecies], *cn[kMaxSpecies], *b[kMaxSpecies], *diag[kMaxSpecies];
     float *diag32[kMaxSpecies];
     int32_t *err;
@@ -67,8 +69,9 @@ struct GuardBand {
 // kTab: the device-resident form (rows from the rate tables; tile coordinates
 // and tables written earlier in the same kernel, so read through L2).
 // gb (device-resident step): a tumour voxel in the guard band sets *hit.
-template <bool kTab>
-__device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, int64_t e, const RowTab *tab = nullptr,
+// kVar: the lattice has a diffusivity factor per voxel.
+template <bool kTab, bool kVar>
+__device__ __forceinline__ void prep_elem_t(const BatchSys &S, const BoxGeo &g, int64_t e, const RowTab *tab = nullptr,
                                           const GuardBand *gb = nullptr, bool *hit = nullptr)
 {
     const int ns = S.C.nspecies;
@@ -76,7 +79,9 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
     if (!elem_box<kTab>(e, g, S.tile_coord, bx, by, bz)) {   // tile padding
         S.flags[e] = 0;
         S.cell[e] = 0;
-        if (S.dfac) S.dfac[e] = 1.0;
+        if (kVar) S.dfac[e] = 1.0;
+        if (kVar && S.hm)
+            for (int d = 0; d < 6; ++d) S.hm[d * S.hstride + e] = 0.0;
         for (int s = 0; s < ns; ++s) {
             S.x[s][e] = 0.0;
             S.cn[s][e] = 0.0;
@@ -100,7 +105,7 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
     const uint32_t m5 = hz0 ? __ldg(S.mask + L - sz) : 0u, m6 = hz1 ? __ldg(S.mask + L + sz) : 0u;
     const int32_t id0 = __ldg(S.cell_id + L);
     if (gb && id0 > 0 && gb->in(bx, by, bz, g)) *hit = true;
-    const double fp = S.dfac_lat ? __ldg(S.dfac_lat + L) : 1.0;
+    const double fp = kVar ? __ldg(S.dfac_lat + L) : 1.0;
     double cs[kMaxSpecies];
 #pragma unroll
     for (int s = 0; s < kMaxSpecies; ++s) cs[s] = s < ns ? __ldg(S.field[s] + L) : 0.0;
@@ -119,7 +124,7 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
     const int32_t id = bad ? 0 : id0;
     // the rate-table entries of the cell id, every species together
     double dkv[kMaxSpecies], dqv[kMaxSpecies];
-    const bool tabrow = kTab && !S.dfac && inm;
+    const bool tabrow = kTab && !kVar && inm;
 #pragma unroll
     for (int s = 0; s < kMaxSpecies; ++s) {
         const int64_t k = (int64_t)s * S.C.ncell + id;
@@ -128,9 +133,11 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
     }
     S.flags[e] = (uint8_t)f;
     S.cell[e] = id0;
-    if (S.dfac) S.dfac[e] = fp;
+    if (kVar) S.dfac[e] = fp;
     if (bad) atomicOr(S.err, 1);
     if (!inm) {                                 // identity row keeping c^n
+        if (kVar && S.hm)
+            for (int d = 0; d < 6; ++d) S.hm[d * S.hstride + e] = 0.0;
 #pragma unroll
         for (int s = 0; s < kMaxSpecies; ++s) {
             if (s >= ns) break;
@@ -150,6 +157,13 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
         const int64_t o = d == 0 ? -1 : d == 1 ? 1 : d == 2 ? -sy : d == 3 ? sy : d == 4 ? -sz : sz;
         return __ldg(S.dfac_lat + L + o);
     };
+    double hm[6], hsum = 0.0;
+    if (kVar) {
+        hsum = face_means(f, fp, dq, hm);
+        if (S.hm)
+#pragma unroll
+            for (int d = 0; d < 6; ++d) S.hm[d * S.hstride + e] = hm[d];
+    }
 #pragma unroll
     for (int s = 0; s < kMaxSpecies; ++s) {
         if (s >= ns) break;
@@ -161,7 +175,7 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
             dg = dkv[s] + tab->aDn[s][__popc(f & F_OPEN) + 2 * ndir];
             bb = (c + dqv[s]) + tab->wbn[s][ndir];
         } else {
-            assemble_row(S.C, s, f, id, ndir, S.dfac != nullptr, fp, dq, c, dg, bb);
+            assemble_row(S.C, s, f, id, ndir, kVar, fp, hsum, c, dg, bb);
         }
         S.x[s][e] = c;
         S.cn[s][e] = c;
@@ -169,6 +183,14 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
         S.diag32[s][e] = f32_rz(dg);
         S.b[s][e] = bb;
     }
+}
+
+template <bool kTab>
+__device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, int64_t e, const RowTab *tab = nullptr,
+                                          const GuardBand *gb = nullptr, bool *hit = nullptr)
+{
+    if (S.dfac) prep_elem_t<kTab, true>(S, g, e, tab, gb, hit);
+    else prep_elem_t<kTab, false>(S, g, e, tab, gb, hit);
 }
 
 // The device-resident preparation for uniform D on tiles at least four wide
@@ -398,7 +420,7 @@ __device__ __forceinline__ GuardBand guard_band(const ExtractArgs &A, const BoxG
 // Phase E: gather + rows of every stored element (4-element chunks where the
 // tiles are at least four wide and D is uniform), the neighbour table when
 // nbr, and with kGuard the guard vote (one atomic per CTA).
-template <int NT, bool kGuard>
+template <int NT, bool kGuard, bool VAR>
 __device__ __forceinline__ void gather_phase_t(const ExtractArgs &A, const BatchSys &S, const BoxGeo &g, int64_t NE,
                                                int b, int nb, const RowTab &tab, bool nbr)
 {
@@ -407,12 +429,13 @@ __device__ __forceinline__ void gather_phase_t(const ExtractArgs &A, const Batch
     const GuardBand gbv = guard_band(A, g);
     const GuardBand *gb = kGuard ? &gbv : nullptr;
     bool hit = false;
-    const bool chunks = g.lt[0] >= 2 && !S.dfac;
+    const bool chunks = g.lt[0] >= 2 && !(VAR && S.dfac);
     const int64_t nunit = chunks ? NE >> 2 : NE;   // 4-element chunks or elements
     for (int64_t u = (int64_t)b * NT + tid; u < nunit; u += (int64_t)nb * NT) {
         const int64_t e = chunks ? u << 2 : u;
         if (chunks) prep_chunk(S, g, (uint32_t)u, &tab, gb, &hit);
-        else prep_elem<true>(S, g, e, &tab, gb, &hit);
+        else if (VAR) prep_elem<true>(S, g, e, &tab, gb, &hit);
+        else prep_elem_t<true, false>(S, g, e, &tab, gb, &hit);
         if (nbr && (e & ((1 << ltv) - 1)) == 0) {   // neighbour tiles of this tile
             const int64_t a = e >> ltv;
             const int4 c = __ldcg(reinterpret_cast<const int4 *>(S.tile_coord) + a);
@@ -430,12 +453,12 @@ __device__ __forceinline__ void gather_phase_t(const ExtractArgs &A, const Batch
     if (kGuard && __syncthreads_or(hit) && tid == 0) atomicOr(&A.cad->guard_hit, 1u);
 }
 
-template <int NT>
+template <int NT, bool VAR>
 __device__ __forceinline__ void gather_phase(const ExtractArgs &A, const BatchSys &S, const BoxGeo &g, int64_t NE,
                                              int b, int nb, const RowTab &tab, bool nbr)
 {
-    if (A.box_every > 1 && A.box_guard > 0) gather_phase_t<NT, true>(A, S, g, NE, b, nb, tab, nbr);
-    else gather_phase_t<NT, false>(A, S, g, NE, b, nb, tab, nbr);
+    if (A.box_every > 1 && A.box_guard > 0) gather_phase_t<NT, true, VAR>(A, S, g, NE, b, nb, tab, nbr);
+    else gather_phase_t<NT, false, VAR>(A, S, g, NE, b, nb, tab, nbr);
 }
 
 // Block-wide sum over NT threads (every thread gets the total).
@@ -467,7 +490,7 @@ __device__ __forceinline__ unsigned long long xblock_sum(unsigned long long v, u
 //   E  the gather and rows of every stored element (Eq. 1-4) and the tile
 //      neighbour table; CTA 0 then publishes the box and element count.
 // Returns false when a grid barrier gave up (A.xabort is then set).
-template <int NT>
+template <int NT, bool VAR>
 __device__ __forceinline__ bool extract_phases(const ExtractArgs &A, const BatchSys &S, int b, int nb,
                                                uint32_t &epoch)
 {
@@ -732,7 +755,7 @@ __device__ __forceinline__ bool extract_phases(const ExtractArgs &A, const Batch
     for (int32_t wi = w0 + tid; wi < w1; wi += NT) aw[wi] = 0ull;
     const int ltv = g.lt[0] + g.lt[1] + g.lt[2];
     const int64_t NE = g.n[0] > 0 ? nact << ltv : 0;
-    gather_phase<NT>(A, S, g, NE, b, nb, tab, true);
+    gather_phase<NT, VAR>(A, S, g, NE, b, nb, tab, true);
     if (b == 0 && tid == 0) {
         A.dyn->g = g;
         A.dyn->NE = NE;
@@ -744,7 +767,7 @@ __device__ __forceinline__ bool extract_phases(const ExtractArgs &A, const Batch
 // A step that keeps the box, tiles and neighbour table of the last full
 // extraction (box_every > 1): the resets the compaction does, the row and rate
 // tables, one grid barrier, then the gather + rows of every stored element.
-template <int NT>
+template <int NT, bool VAR>
 __device__ __forceinline__ bool refresh_phases(const ExtractArgs &A, const BatchSys &S, int b, int nb, uint32_t &epoch)
 {
     __shared__ RowTab tab;
@@ -764,7 +787,7 @@ __device__ __forceinline__ bool refresh_phases(const ExtractArgs &A, const Batch
     if (!team_barrier(A.bar, epoch, nb, A.xabort, A.timeout_ns)) return false;
     const BoxGeo g = A.dyn->g;
     const int64_t NE = A.dyn->NE;
-    gather_phase<NT>(A, S, g, NE, b, nb, tab, false);
+    gather_phase<NT, VAR>(A, S, g, NE, b, nb, tab, false);
     if (prof) A.prof[14] += globaltimer_ns() - tp;
     return true;
 }

@@ -20,7 +20,6 @@
 
 #include "mpm_internal.cuh"
 
-int mpm_solver_max_blocks(mpm_ctx *ctx, int prec, int m, int variant);
 int mpm_solver_variants(int prec, int m);
 
 namespace {
