@@ -882,6 +882,8 @@ static mpm_status enqueue_step(mpm_ctx *ctx, StepGraph *T, mpm_subgrid *sub, con
     for (int d = 0; d < 3; ++d) { X.L[d] = lat->dims[d]; X.lt[d] = sub->lt[d]; }
     X.margin = margin;
     X.vec4 = ((uintptr_t)lat->cell_id % 16) == 0;
+    X.vec = X.vec4 && lat->dims[0] % 4 == 0 && (uintptr_t)lat->mask % 4 == 0;
+    for (int s = 0; s < prm->nspecies; ++s) X.vec = X.vec && (uintptr_t)lat->field[s] % 32 == 0;
     X.part_box = (int32_t *)T->d_xscr;
     X.part_cnt = (unsigned long long *)(T->d_xscr + (size_t)nb * 32);
     X.bar = (uint32_t *)(T->d_xscr + (size_t)nb * 48);

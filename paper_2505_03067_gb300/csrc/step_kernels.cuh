@@ -199,13 +199,43 @@ __device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, in
 // lattice loads of all four are in flight together, and the element arrays
 // are written with 4- to 16-byte stores.  Per element the rows are those of
 // prep_elem<true> (same operands, same order).
-__device__ __forceinline__ void prep_chunk(const BatchSys &S, const BoxGeo &g, uint32_t r, const RowTab *tab,
-                                           const GuardBand *gb, bool *hit)
+//
+// Lattice reads.  The lanes of a warp lie in 32 different lattice rows, so every
+// load instruction costs 32 look-ups in L1 whatever its width, and those
+// look-ups bound the phase (38 loads an element chunk, a word or less each:
+// 112 us for 2.8 M stored elements).  A box starts at any x, but its chunks
+// start at x = lo mod 4 everywhere: with kAl = lo & 3 known (kAl >= 0: rows of
+// a multiple of 4 voxels, arrays aligned) a chunk's four mask bytes, ids or
+// fields are cut from one or two aligned words, 16-byte or 32-byte vectors
+// (18 loads: 100 us); kAl < 0 is the form for other lattices.
+__device__ __forceinline__ void ld4_f64(const double *p, double (&v)[4])
+{
+    asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(v[0]), "=d"(v[1]), "=d"(v[2]), "=d"(v[3]) : "l"(p));
+}
+__device__ __forceinline__ void st4_f64(double *p, const double (&v)[4])
+{
+    asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(v[0]), "d"(v[1]), "d"(v[2]), "d"(v[3])
+                 : "memory");
+}
+
+// The mask bytes x0 .. x0 + 3 of a lattice row (row: its first byte), where x0 =
+// kAl mod 4; more: the word after the first holds voxels of the row.
+template <int kAl>
+__device__ __forceinline__ uint32_t mask4(const uint8_t *row, int x0, bool more)
+{
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(row + (x0 - kAl));
+    const uint32_t lo = __ldg(w);
+    if (kAl == 0) return lo;
+    return __funnelshift_r(lo, more ? __ldg(w + 1) : 0u, 8 * kAl);
+}
+
+template <int kAl>
+__device__ __forceinline__ void prep_chunk(const BatchSys &S, const BoxGeo &g, uint32_t r, const int4 tc,
+                                           const RowTab *tab, const GuardBand *gb, bool *hit)
 {
     const int ns = S.C.nspecies;
     const uint32_t e = r << 2;
     const int ltv = g.lt[0] + g.lt[1] + g.lt[2];
-    const int4 tc = __ldcg(reinterpret_cast<const int4 *>(S.tile_coord) + (e >> ltv));
     const uint32_t v0 = e & ((1u << ltv) - 1u);
     const int ix0 = (int)(v0 & ((1u << g.lt[0]) - 1u));
     const int iy = (int)((v0 >> g.lt[0]) & ((1u << g.lt[1]) - 1u)), iz = (int)(v0 >> (g.lt[0] + g.lt[1]));
@@ -217,26 +247,67 @@ __device__ __forceinline__ void prep_chunk(const BatchSys &S, const BoxGeo &g, u
     uint32_t mo[4], my0[4], my1[4], mz0[4], mz1[4];
     int32_t id0[4];
     double cs[kMaxSpecies][4];
+    uint32_t mxm = 0u, mxp = 0u;
+    if (kAl >= 0) {
+        constexpr int A = kAl < 0 ? 0 : kAl;
+        const bool in = nv > 0;
+        const int x0 = g.lo[0] + bx0;
+        const bool more = x0 - A + 4 < (int)g.Lx;   // whole vectors: the row is a multiple of 4 long
+        const uint8_t *row = S.mask + (L0 - x0);
+        const uint32_t wo = in ? mask4<A>(row, x0, more) : 0u;
+        const uint32_t wy0 = in && hy0 ? mask4<A>(row - sy, x0, more) : 0u;
+        const uint32_t wy1 = in && hy1 ? mask4<A>(row + sy, x0, more) : 0u;
+        const uint32_t wz0 = in && hz0 ? mask4<A>(row - sz, x0, more) : 0u;
+        const uint32_t wz1 = in && hz1 ? mask4<A>(row + sz, x0, more) : 0u;
+        if (in && bx0 > 0) mxm = __ldg(row + x0 - 1);
+        if (nv == 4 && bx0 + 4 < g.n[0]) mxp = __ldg(row + x0 + 4);
+        const int4 *ip = reinterpret_cast<const int4 *>(S.cell_id + (L0 - A));
+        int4 i0 = make_int4(0, 0, 0, 0), i1 = i0;
+        if (in) i0 = __ldg(ip);
+        if (A > 0 && in && more) i1 = __ldg(ip + 1);
+        const int32_t iv[8] = {i0.x, i0.y, i0.z, i0.w, i1.x, i1.y, i1.z, i1.w};
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const bool in = k < nv;
-        const int64_t L = L0 + k;
-        mo[k] = in ? __ldg(S.mask + L) : 0u;
-        my0[k] = in && hy0 ? __ldg(S.mask + L - sy) : 0u;
-        my1[k] = in && hy1 ? __ldg(S.mask + L + sy) : 0u;
-        mz0[k] = in && hz0 ? __ldg(S.mask + L - sz) : 0u;
-        mz1[k] = in && hz1 ? __ldg(S.mask + L + sz) : 0u;
-        id0[k] = in ? __ldg(S.cell_id + L) : 0;
+        for (int s = 0; s < kMaxSpecies; ++s) {
+            double f0[4] = {0.0, 0.0, 0.0, 0.0}, f1[4] = {0.0, 0.0, 0.0, 0.0};
+            if (s < ns && in) {
+                ld4_f64(S.field[s] + (L0 - A), f0);
+                if (A > 0 && more) ld4_f64(S.field[s] + (L0 - A) + 4, f1);
+            }
 #pragma unroll
-        for (int s = 0; s < kMaxSpecies; ++s) cs[s][k] = in && s < ns ? __ldg(S.field[s] + L) : 0.0;
+            for (int k = 0; k < 4; ++k) cs[s][k] = k < nv ? (k + A < 4 ? f0[(k + A) & 3] : f1[(k + A) & 3]) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const uint32_t keep = k < nv ? 0xffu : 0u;
+            mo[k] = (wo >> (8 * k)) & keep;
+            my0[k] = (wy0 >> (8 * k)) & keep;
+            my1[k] = (wy1 >> (8 * k)) & keep;
+            mz0[k] = (wz0 >> (8 * k)) & keep;
+            mz1[k] = (wz1 >> (8 * k)) & keep;
+            id0[k] = k < nv ? iv[k + A] : 0;
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const bool in = k < nv;
+            const int64_t L = L0 + k;
+            mo[k] = in ? __ldg(S.mask + L) : 0u;
+            my0[k] = in && hy0 ? __ldg(S.mask + L - sy) : 0u;
+            my1[k] = in && hy1 ? __ldg(S.mask + L + sy) : 0u;
+            mz0[k] = in && hz0 ? __ldg(S.mask + L - sz) : 0u;
+            mz1[k] = in && hz1 ? __ldg(S.mask + L + sz) : 0u;
+            id0[k] = in ? __ldg(S.cell_id + L) : 0;
+#pragma unroll
+            for (int s = 0; s < kMaxSpecies; ++s) cs[s][k] = in && s < ns ? __ldg(S.field[s] + L) : 0.0;
+        }
+        mxm = nv > 0 && bx0 > 0 ? __ldg(S.mask + L0 - 1) : 0u;
+        mxp = nv == 4 && bx0 + 4 < g.n[0] ? __ldg(S.mask + L0 + 4) : 0u;
     }
     if (gb) {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (k < nv && id0[k] > 0 && gb->in(bx0 + k, by, bz, g)) *hit = true;
     }
-    const uint32_t mxm = nv > 0 && bx0 > 0 ? __ldg(S.mask + L0 - 1) : 0u;
-    const uint32_t mxp = nv == 4 && bx0 + 4 < g.n[0] ? __ldg(S.mask + L0 + 4) : 0u;
     uint32_t f[4];
     int32_t id[4];
     int nd[4];
@@ -274,9 +345,11 @@ __device__ __forceinline__ void prep_chunk(const BatchSys &S, const BoxGeo &g, u
             const int64_t t = (int64_t)s * S.C.ncell + id[k];
             const bool row = (f[k] & F_MASK) != 0;
             // plain cached loads: the tables were written before a grid barrier
-            // and never read before it, and neighbouring voxels mostly share a cell
-            dkv[k] = row ? S.dk[t] : 0.0;
-            dqv[k] = row ? S.dq[t] : 0.0;
+            // and never read before it.  Neighbouring voxels mostly share a
+            // cell: its entries are not looked up again.
+            const bool same = k > 0 && (f[k - (k > 0)] & F_MASK) && id[k] == id[k - (k > 0)];
+            dkv[k] = row ? (same ? dkv[k - (k > 0)] : S.dk[t]) : 0.0;
+            dqv[k] = row ? (same ? dqv[k - (k > 0)] : S.dq[t]) : 0.0;
         }
         double xo[4], dg[4], bb[4];
         float d32[4];
@@ -298,16 +371,10 @@ __device__ __forceinline__ void prep_chunk(const BatchSys &S, const BoxGeo &g, u
             }
             d32[k] = f32_rz(dg[k]);
         }
-        double2 *x2 = reinterpret_cast<double2 *>(S.x[s] + e), *c2 = reinterpret_cast<double2 *>(S.cn[s] + e);
-        double2 *b2 = reinterpret_cast<double2 *>(S.b[s] + e), *g2 = reinterpret_cast<double2 *>(S.diag[s] + e);
-        x2[0] = make_double2(xo[0], xo[1]);
-        x2[1] = make_double2(xo[2], xo[3]);
-        c2[0] = make_double2(xo[0], xo[1]);
-        c2[1] = make_double2(xo[2], xo[3]);
-        b2[0] = make_double2(bb[0], bb[1]);
-        b2[1] = make_double2(bb[2], bb[3]);
-        g2[0] = make_double2(dg[0], dg[1]);
-        g2[1] = make_double2(dg[2], dg[3]);
+        st4_f64(S.x[s] + e, xo);
+        st4_f64(S.cn[s] + e, xo);
+        st4_f64(S.b[s] + e, bb);
+        st4_f64(S.diag[s] + e, dg);
         *reinterpret_cast<float4 *>(S.diag32[s] + e) = make_float4(d32[0], d32[1], d32[2], d32[3]);
     }
 }
@@ -365,6 +432,7 @@ struct ExtractArgs {
     const int32_t *cell_id;
     const uint8_t *mask;
     int32_t L[3], lt[3], margin, vec4;
+    int32_t vec;                       // Lx a multiple of 4, mask, ids and fields aligned for 4-voxel vectors
     int32_t *part_box;                 // [grid][8]: per-CTA min[3], max[3]
     unsigned long long *part_cnt;      // [grid][2]: per-CTA mask voxels, active tiles
     uint32_t *bar;                     // grid barrier counter (zero at launch)
@@ -419,26 +487,32 @@ __device__ __forceinline__ GuardBand guard_band(const ExtractArgs &A, const BoxG
 
 // Phase E: gather + rows of every stored element (4-element chunks where the
 // tiles are at least four wide and D is uniform), the neighbour table when
-// nbr, and with kGuard the guard vote (one atomic per CTA).
-template <int NT, bool kGuard, bool VAR>
+// nbr, and with a guard band the guard vote (one atomic per CTA).
+template <int NT, bool VAR, int kAl>
 __device__ __forceinline__ void gather_phase_t(const ExtractArgs &A, const BatchSys &S, const BoxGeo &g, int64_t NE,
                                                int b, int nb, const RowTab &tab, bool nbr)
 {
     const int tid = threadIdx.x;
     const int ltv = g.lt[0] + g.lt[1] + g.lt[2];
     const GuardBand gbv = guard_band(A, g);
-    const GuardBand *gb = kGuard ? &gbv : nullptr;
+    const bool guard = A.box_every > 1 && A.box_guard > 0;
+    const GuardBand *gb = guard ? &gbv : nullptr;
     bool hit = false;
     const bool chunks = g.lt[0] >= 2 && !(VAR && S.dfac);
     const int64_t nunit = chunks ? NE >> 2 : NE;   // 4-element chunks or elements
-    for (int64_t u = (int64_t)b * NT + tid; u < nunit; u += (int64_t)nb * NT) {
+    const int64_t u0 = (int64_t)b * NT + tid, us = (int64_t)nb * NT;
+    const int lu = chunks ? ltv - 2 : ltv;
+    const int4 *tcs = reinterpret_cast<const int4 *>(S.tile_coord);
+    int4 next = u0 < nunit ? __ldcg(tcs + (u0 >> lu)) : make_int4(0, 0, 0, 0);   // a tile ahead
+    for (int64_t u = u0; u < nunit; u += us) {
         const int64_t e = chunks ? u << 2 : u;
-        if (chunks) prep_chunk(S, g, (uint32_t)u, &tab, gb, &hit);
+        const int4 c = next;
+        if (u + us < nunit) next = __ldcg(tcs + ((u + us) >> lu));
+        if (chunks) prep_chunk<kAl>(S, g, (uint32_t)u, c, &tab, gb, &hit);
         else if (VAR) prep_elem<true>(S, g, e, &tab, gb, &hit);
         else prep_elem_t<true, false>(S, g, e, &tab, gb, &hit);
         if (nbr && (e & ((1 << ltv) - 1)) == 0) {   // neighbour tiles of this tile
             const int64_t a = e >> ltv;
-            const int4 c = __ldcg(reinterpret_cast<const int4 *>(S.tile_coord) + a);
 #pragma unroll
             for (int d = 0; d < 6; ++d) {
                 int32_t q[3] = {c.x, c.y, c.z};
@@ -450,15 +524,20 @@ __device__ __forceinline__ void gather_phase_t(const ExtractArgs &A, const Batch
             }
         }
     }
-    if (kGuard && __syncthreads_or(hit) && tid == 0) atomicOr(&A.cad->guard_hit, 1u);
+    if (guard && __syncthreads_or(hit) && tid == 0) atomicOr(&A.cad->guard_hit, 1u);
 }
 
 template <int NT, bool VAR>
 __device__ __forceinline__ void gather_phase(const ExtractArgs &A, const BatchSys &S, const BoxGeo &g, int64_t NE,
                                              int b, int nb, const RowTab &tab, bool nbr)
 {
-    if (A.box_every > 1 && A.box_guard > 0) gather_phase_t<NT, true, VAR>(A, S, g, NE, b, nb, tab, nbr);
-    else gather_phase_t<NT, false, VAR>(A, S, g, NE, b, nb, tab, nbr);
+    switch (A.vec ? g.lo[0] & 3 : -1) {
+    case 0: gather_phase_t<NT, VAR, 0>(A, S, g, NE, b, nb, tab, nbr); break;
+    case 1: gather_phase_t<NT, VAR, 1>(A, S, g, NE, b, nb, tab, nbr); break;
+    case 2: gather_phase_t<NT, VAR, 2>(A, S, g, NE, b, nb, tab, nbr); break;
+    case 3: gather_phase_t<NT, VAR, 3>(A, S, g, NE, b, nb, tab, nbr); break;
+    default: gather_phase_t<NT, VAR, -1>(A, S, g, NE, b, nb, tab, nbr);
+    }
 }
 
 // Block-wide sum over NT threads (every thread gets the total).
@@ -610,36 +689,89 @@ __device__ __forceinline__ bool extract_phases(const ExtractArgs &A, const Batch
         __syncthreads();
         unsigned long long cnt = 0;
         if (g.n[0] > 0) {
-            // one row of tiles (TY x TZ box rows) per warp and iteration: for
-            // each 32-voxel chunk the mask bytes of those rows are in flight
-            // together and OR-ed, and the chunk's active tiles are written
-            // once, by the first lane of each tile (the rows of a tile would
-            // otherwise store the same activity bytes again and again)
             const int64_t gw = (int64_t)b * (NT / 32) + warp, nw = (int64_t)nb * (NT / 32);
             const int TX = 1 << g.lt[0], TY = 1 << g.lt[1], TZ = 1 << g.lt[2];
             const int64_t ngroups = (int64_t)g.nt[1] * g.nt[2];
-            for (int64_t grp = gw; grp < ngroups; grp += nw) {
-                const int ty = (int)(grp % g.nt[1]), tz = (int)(grp / g.nt[1]);
-                const int64_t trow = ((int64_t)tz * g.nt[1] + ty) * g.nt[0];
-                const int y1 = min(TY, g.n[1] - ty * TY), z1 = min(TZ, g.n[2] - tz * TZ);
-                const int nr = y1 * z1;
-                for (int c0 = 0; c0 < g.n[0]; c0 += 32) {
-                    const int bx = c0 + lane;
+            if (A.vec) {
+                // 128 voxels of one row of tiles (TY x TZ box rows) per warp and
+                // iteration, four voxels a lane: a box row's four bytes are cut
+                // from two aligned words, eight rows' words are in flight, and
+                // their OR gives the tiles' activity.  Bound by the latency of
+                // those loads: 55 -> 21 us for a box of 20 M voxels, against
+                // one byte a lane.
+                const int al = g.lo[0] & 3, end = g.lo[0] + g.n[0];
+                const uint32_t nch = ((uint32_t)g.n[0] + 127u) / 128u, nty = (uint32_t)g.nt[1];
+                const uint32_t items = (uint32_t)ngroups * nch;
+                for (uint32_t it = (uint32_t)gw; it < items; it += (uint32_t)nw) {
+                    const uint32_t grp = it / nch, ch = it - grp * nch;
+                    const int tz = (int)(grp / nty), ty = (int)(grp - (uint32_t)tz * nty);
+                    const int bx = (int)(ch * 128u) + 4 * lane;     // box x of the lane's four voxels
+                    const int xa = g.lo[0] + bx - al;               // its first word
+                    const bool w0 = bx < g.n[0], w1 = al > 0 && w0 && xa + 4 < end;
+                    const uint32_t keep = !w0 ? 0u : g.n[0] - bx >= 4 ? 0xffffffffu : (1u << (8 * (g.n[0] - bx))) - 1u;
                     uint32_t any = 0u;
-                    if (bx < g.n[0]) {
-#pragma unroll 4
-                        for (int r = 0; r < nr; ++r) {
-                            const int by = ty * TY + r % y1, bz = tz * TZ + r / y1;
-                            const int64_t L0 = (int64_t)g.lo[0] +
-                                               (int64_t)g.Lx * ((int64_t)(g.lo[1] + by) + (int64_t)g.Ly * (g.lo[2] + bz));
-                            const uint32_t m = __ldg(A.mask + L0 + bx);
-                            cnt += m != 0u ? 1u : 0u;
-                            any |= m;
+                    const int nr = TY * TZ;
+                    for (int r0 = 0; r0 < nr; r0 += 8) {
+                        uint32_t lo[8], hi[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const int r = r0 + q;
+                            const int by = ty * TY + (r & (TY - 1)), bz = tz * TZ + (r >> g.lt[1]);
+                            const bool in = r < nr && by < g.n[1] && bz < g.n[2];
+                            const uint32_t *p = reinterpret_cast<const uint32_t *>(
+                                A.mask + (int64_t)g.Lx * ((int64_t)(g.lo[1] + by) + (int64_t)g.Ly * (g.lo[2] + bz)) + xa);
+                            lo[q] = in && w0 ? __ldg(p) : 0u;
+                            hi[q] = in && w1 ? __ldg(p + 1) : 0u;
+                        }
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const uint32_t m = __funnelshift_r(lo[q], hi[q], 8 * al) & keep;
+                            const uint32_t nz = (((m & 0x7f7f7f7fu) + 0x7f7f7f7fu) | m) & 0x80808080u;
+                            cnt += __popc(nz);
+                            any |= nz;
                         }
                     }
-                    const unsigned bal = __ballot_sync(0xffffffffu, any != 0u);
-                    if ((lane & (TX - 1)) == 0 && ((bal >> lane) & ((TX >= 32) ? 0xffffffffu : ((1u << TX) - 1u))))
-                        A.active[trow + (bx >> g.lt[0])] = 1;
+                    const int64_t trow = ((int64_t)tz * g.nt[1] + ty) * g.nt[0];
+                    if (TX >= 4) {
+                        const int G = TX >> 2;          // lanes of a tile
+                        const unsigned bal = __ballot_sync(0xffffffffu, any != 0u);
+                        if ((lane & (G - 1)) == 0 && ((bal >> lane) & ((1u << G) - 1u)))
+                            A.active[trow + (bx >> g.lt[0])] = 1;
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)     // a lane's four voxels: two or four tiles
+                            if ((any >> (8 * k)) & 0x80u) A.active[trow + ((bx + k) >> g.lt[0])] = 1;
+                    }
+                }
+            } else {
+                // one row of tiles (TY x TZ box rows) per warp and iteration: for
+                // each 32-voxel chunk the mask bytes of those rows are in flight
+                // together and OR-ed, and the chunk's active tiles are written
+                // once, by the first lane of each tile (the rows of a tile would
+                // otherwise store the same activity bytes again and again)
+                for (int64_t grp = gw; grp < ngroups; grp += nw) {
+                    const int ty = (int)(grp % g.nt[1]), tz = (int)(grp / g.nt[1]);
+                    const int64_t trow = ((int64_t)tz * g.nt[1] + ty) * g.nt[0];
+                    const int y1 = min(TY, g.n[1] - ty * TY), z1 = min(TZ, g.n[2] - tz * TZ);
+                    const int nr = y1 * z1;
+                    for (int c0 = 0; c0 < g.n[0]; c0 += 32) {
+                        const int bx = c0 + lane;
+                        uint32_t any = 0u;
+                        if (bx < g.n[0]) {
+#pragma unroll 4
+                            for (int r = 0; r < nr; ++r) {
+                                const int by = ty * TY + r % y1, bz = tz * TZ + r / y1;
+                                const int64_t L0 = (int64_t)g.lo[0] +
+                                                   (int64_t)g.Lx * ((int64_t)(g.lo[1] + by) + (int64_t)g.Ly * (g.lo[2] + bz));
+                                const uint32_t m = __ldg(A.mask + L0 + bx);
+                                cnt += m != 0u ? 1u : 0u;
+                                any |= m;
+                            }
+                        }
+                        const unsigned bal = __ballot_sync(0xffffffffu, any != 0u);
+                        if ((lane & (TX - 1)) == 0 && ((bal >> lane) & ((TX >= 32) ? 0xffffffffu : ((1u << TX) - 1u))))
+                            A.active[trow + (bx >> g.lt[0])] = 1;
+                    }
                 }
             }
         }
