@@ -515,10 +515,11 @@ __device__ __forceinline__ bool use_rows(const SysDev &S)
 // element the operands and the order of the sum are those of the scalar pass,
 // so w is the same bit for bit; the dot products add four elements per thread
 // and iteration.  Vectors written during the solve are read through L2.
-template <typename T, int MAXM, int LIM = MAXM>
-__device__ __forceinline__ void pass_arnoldi1_rows(const SysDev &S, int j, T sj, uint32_t e0, uint32_t es,
+template <typename T, int MAXM, int LIM = MAXM, int JJ = -1>
+__device__ __forceinline__ void pass_arnoldi1_rows(const SysDev &S, int jr, T sj, uint32_t e0, uint32_t es,
                                                    T (&acc)[MAXM + 1], bool want_ww)
 {
+    const int j = JJ >= 0 ? JJ : jr;   // JJ >= 0: the step index known at compile time
     const uint32_t NR = (uint32_t)S.NE >> 2;
     const int64_t vs = S.vstride;
     const T offT = (T)S.off[0];
@@ -527,13 +528,26 @@ __device__ __forceinline__ void pass_arnoldi1_rows(const SysDev &S, int j, T sj,
     const T *dgp = diag_of<T>(S, 0);
     const int ltx = S.ltx, lty = S.lty, ltv = S.ltx + S.lty + S.ltz;
     const uint32_t TX = 1u << ltx, TY = 1u << lty, TZ = 1u << S.ltz, TXY = TX * TY;
+    // the neighbour entries and flags of a chunk are fetched one chunk ahead, so
+    // that its stencil loads never wait for them
+    int32_t nn[6] = {0, 0, 0, 0, 0, 0};
+    uchar4 fn = make_uchar4(0, 0, 0, 0);
+    if (e0 < NR) {
+        tile_nbrs(S.nbr, e0 << 2, ltv, nn);
+        fn = ldro(reinterpret_cast<const uchar4 *>(S.flags) + e0);
+    }
     for (uint32_t r = e0; r < NR; r += es) {
         const uint32_t e = r << 2;
         const uint32_t v0 = e & ((1u << ltv) - 1u);
         const uint32_t ix0 = v0 & (TX - 1), iy = (v0 >> ltx) & (TY - 1), iz = v0 >> (ltx + lty);
         int32_t tn[6];
-        tile_nbrs(S.nbr, e, ltv, tn);
-        const uchar4 fl = ldro(reinterpret_cast<const uchar4 *>(S.flags) + r);
+#pragma unroll
+        for (int d = 0; d < 6; ++d) tn[d] = nn[d];
+        const uchar4 fl = fn;
+        if (r + es < NR) {
+            tile_nbrs(S.nbr, (r + es) << 2, ltv, nn);
+            fn = ldro(reinterpret_cast<const uchar4 *>(S.flags) + r + es);
+        }
         // element of the neighbour tile across face d at offset o, or e when
         // there is none (every face that way is then closed)
         auto other = [&](int d, uint32_t o) -> uint32_t { return tn[d] >= 0 ? ((uint32_t)tn[d] << ltv) + o : e; };
@@ -547,6 +561,13 @@ __device__ __forceinline__ void pass_arnoldi1_rows(const SysDev &S, int j, T sj,
         const Q4<T> ym = ld4cg(uj + qym), yp = ld4cg(uj + qyp), zm = ld4cg(uj + qzm), zp = ld4cg(uj + qzp);
         const T xm = __ldcg(uj + qxm), xp = __ldcg(uj + qxp);
         const Q4<T> dg = ld4ro(dgp + e);
+        // the basis rows travel with the stencil's where the step index is known
+        // (else their registers, for LIM vectors, would spill)
+        Q4<T> vb[JJ > 0 ? JJ : 1];
+        if (JJ > 0) {
+#pragma unroll
+            for (int i = 0; i < JJ; ++i) vb[i] = ld4cg(V + (int64_t)i * vs + e);
+        }
         const uint32_t ff[4] = {fl.x, fl.y, fl.z, fl.w};
         T w[4];
 #pragma unroll
@@ -561,7 +582,7 @@ __device__ __forceinline__ void pass_arnoldi1_rows(const SysDev &S, int j, T sj,
 #pragma unroll
         for (int i = 0; i < LIM; ++i) {
             if (i < j) {
-                const Q4<T> b = ld4cg(V + (int64_t)i * vs + e);
+                const Q4<T> b = JJ > 0 ? vb[i < JJ ? i : 0] : ld4cg(V + (int64_t)i * vs + e);
                 acc[i] += ((b.v[0] * w[0] + b.v[1] * w[1]) + (b.v[2] * w[2] + b.v[3] * w[3]));
             }
         }
@@ -580,10 +601,12 @@ __device__ __forceinline__ void pass_arnoldi1_form(const SysDev &S, int j, T sj,
 {
     if (exact_j<T, MAXM>())
         with_exact(j, [&](auto J) { pass_arnoldi1_t<T, MAXM, U, FORM, decltype(J)::value>(S, j, sj, e0, es, acc, want_ww); });
+    else if (FORM == D_UNIFORM && MAXM == 8 && use_rows<T>(S))
+        with_exact(j, [&](auto J) { pass_arnoldi1_rows<T, MAXM, MAXM, decltype(J)::value>(S, j, sj, e0, es, acc, want_ww); });
     else
         with_limit<MAXM>(j, [&](auto L) {
             constexpr int LIM = decltype(L)::value;
-            if (FORM == D_UNIFORM && use_rows<T>(S)) pass_arnoldi1_rows<T, MAXM, LIM>(S, j, sj, e0, es, acc, want_ww);
+            if (FORM == D_UNIFORM && MAXM > 8 && use_rows<T>(S)) pass_arnoldi1_rows<T, MAXM, LIM>(S, j, sj, e0, es, acc, want_ww);
             else pass_arnoldi1_t<T, MAXM, U, FORM, -1, LIM>(S, j, sj, e0, es, acc, want_ww);
         });
 }
@@ -626,19 +649,25 @@ __device__ __forceinline__ void pass_arnoldi2_e(const SysDev &S, int jr, const T
     }
 }
 
-template <typename T, int MAXM, int LIM = MAXM>
-__device__ __forceinline__ void pass_arnoldi2_rows(const SysDev &S, int j, const T *c, uint32_t e0, uint32_t es, T &acc)
+template <typename T, int MAXM, int LIM = MAXM, int JJ = -1>
+__device__ __forceinline__ void pass_arnoldi2_rows(const SysDev &S, int jr, const T *c, uint32_t e0, uint32_t es, T &acc)
 {
+    const int j = JJ >= 0 ? JJ : jr;   // JJ >= 0: the step index known at compile time
     const uint32_t NR = (uint32_t)S.NE >> 2;
     const int64_t vs = S.vstride;
     T *V = (T *)S.V[0];
     for (uint32_t r = e0; r < NR; r += es) {
         const uint32_t e = r << 2;
         Q4<T> t = ld4cg(V + (int64_t)(j + 1) * vs + e);
+        Q4<T> vb[JJ >= 0 ? JJ + 1 : 1];   // every load of the chunk before the first product
+        if (JJ >= 0) {
+#pragma unroll
+            for (int i = 0; i <= JJ; ++i) vb[i] = ld4cg(V + (int64_t)i * vs + e);
+        }
 #pragma unroll
         for (int i = 0; i <= LIM; ++i) {
             if (i <= j) {
-                const Q4<T> b = ld4cg(V + (int64_t)i * vs + e);
+                const Q4<T> b = JJ >= 0 ? vb[i <= JJ ? i : 0] : ld4cg(V + (int64_t)i * vs + e);
                 const T ci = c[i];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) t.v[k] -= ci * b.v[k];
@@ -654,10 +683,12 @@ __device__ __forceinline__ void pass_arnoldi2(const SysDev &S, int j, const T *c
 {
     if (exact_j<T, MAXM>() && !use_rows<T>(S))
         with_exact(j, [&](auto J) { pass_arnoldi2_e<T, MAXM, U, decltype(J)::value>(S, j, c, e0, es, acc); });
+    else if (MAXM == 8 && use_rows<T>(S))
+        with_exact(j, [&](auto J) { pass_arnoldi2_rows<T, MAXM, MAXM, decltype(J)::value>(S, j, c, e0, es, acc); });
     else
         with_limit<MAXM>(j, [&](auto L) {
             constexpr int LIM = decltype(L)::value;
-            if (use_rows<T>(S)) pass_arnoldi2_rows<T, MAXM, LIM>(S, j, c, e0, es, acc);
+            if (MAXM > 8 && use_rows<T>(S)) pass_arnoldi2_rows<T, MAXM, LIM>(S, j, c, e0, es, acc);
             else pass_arnoldi2_e<T, MAXM, U, -1, LIM>(S, j, c, e0, es, acc);
         });
 }
@@ -743,9 +774,10 @@ __device__ __forceinline__ void pass_update_e(const SysDev &S, int kr, const T *
     }
 }
 
-template <typename T, int MAXM, int LIM = MAXM>
-__device__ __forceinline__ void pass_update_rows(const SysDev &S, int k, const T *c, uint32_t e0, uint32_t es)
+template <typename T, int MAXM, int LIM = MAXM, int KK = -1>
+__device__ __forceinline__ void pass_update_rows(const SysDev &S, int kr, const T *c, uint32_t e0, uint32_t es)
 {
+    const int k = KK >= 0 ? KK : kr;   // KK >= 0: the vector count known at compile time
     const uint32_t NR = (uint32_t)S.NE >> 2;
     const int64_t vs = S.vstride;
     const T *V = (const T *)S.V[0];
@@ -754,10 +786,15 @@ __device__ __forceinline__ void pass_update_rows(const SysDev &S, int k, const T
         const uint32_t e = r << 2;
         const Q4<double> xv = ld4cg(x + e);
         T d[4] = {T(0), T(0), T(0), T(0)};
+        Q4<T> vb[KK > 0 ? KK : 1];
+        if (KK > 0) {
+#pragma unroll
+            for (int i = 0; i < KK; ++i) vb[i] = ld4cg(V + (int64_t)i * vs + e);
+        }
 #pragma unroll
         for (int i = 0; i < LIM; ++i) {
             if (i < k) {
-                const Q4<T> b = ld4cg(V + (int64_t)i * vs + e);
+                const Q4<T> b = KK > 0 ? vb[i < KK ? i : 0] : ld4cg(V + (int64_t)i * vs + e);
                 const T ci = c[i];
 #pragma unroll
                 for (int q = 0; q < 4; ++q) d[q] += ci * b.v[q];
@@ -775,10 +812,12 @@ __device__ __forceinline__ void pass_update(const SysDev &S, int k, const T *c, 
 {
     if (exact_j<T, MAXM>() && !use_rows<T>(S))   // k = 1..8 vectors
         with_exact(k - 1, [&](auto J) { pass_update_e<T, MAXM, U, decltype(J)::value + 1>(S, k, c, e0, es); });
+    else if (MAXM == 8 && use_rows<T>(S))
+        with_exact(k - 1, [&](auto J) { pass_update_rows<T, MAXM, MAXM, decltype(J)::value + 1>(S, k, c, e0, es); });
     else
         with_limit<MAXM>(k - 1, [&](auto L) {   // i < k <= LIM
             constexpr int LIM = decltype(L)::value;
-            if (use_rows<T>(S)) pass_update_rows<T, MAXM, LIM>(S, k, c, e0, es);
+            if (MAXM > 8 && use_rows<T>(S)) pass_update_rows<T, MAXM, LIM>(S, k, c, e0, es);
             else pass_update_e<T, MAXM, U, -1, LIM>(S, k, c, e0, es);
         });
 }
