@@ -102,15 +102,21 @@ __global__ void k_prep_weights(PrepArgs P)
 }
 
 // The gradient of layer l's weights and bias from the weight-gradient
-// kernel's per-CTA partial sums (summed in CTA order): row m of tap pair p
-// holds (dx copy c, channel ci) = ((c * KC + kc) * 8 + j); the bias row is
-// the ones column (CI = 24: the pad K-column; CI = 16: feature channel 15).
-__global__ void k_wgrad_reduce(const float *__restrict__ partials, int nblk, int CI, int NO, int Ci, int Co,
-                               float *__restrict__ grads)
+// kernel's per-CTA partial sums: row m of tap pair p holds (dx copy c, channel
+// ci) = ((c * KC + kc) * 8 + j); the bias row is the ones column (CI = 24: the
+// pad K-column; CI = 16: feature channel 15).  A CTA takes 32 entries, each
+// warp a range of the partials in CTA order, and the eight ranges are added in
+// order: the sum does not depend on timing.  Bound by the latency of the loads
+// (15 us with one thread per entry, 7 us now, for 24 -> 24 channels).
+__global__ void __launch_bounds__(256) k_wgrad_reduce(const float *__restrict__ partials, int nblk, int CI, int NO,
+                                                      int Ci, int Co, float *__restrict__ grads)
 {
+    __shared__ float s_part[8][32];
     const int KC = CI / 8;
     const int n = 27 * Ci * Co + Co;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    if (i < n) {
         int p, m, co;
         if (i < 27 * Ci * Co) {
             const int t = i / (Ci * Co), ci = (i / Co) % Ci;
@@ -123,8 +129,19 @@ __global__ void k_wgrad_reduce(const float *__restrict__ partials, int nblk, int
             p = 4;
             m = CI == kHC ? 3 * KC * 8 : (KC + 1) * 8 + 7;
         }
+        const int per = (nblk + 7) / 8, b0 = min(nblk, w * per), b1 = min(nblk, b0 + per);
+        const float *src = partials + ((size_t)p * 128 + m) * NO + co;
+        const size_t stride = (size_t)9 * 128 * NO;
         float s = 0.0f;
-        for (int b = 0; b < nblk; ++b) s += partials[(((size_t)b * 9 + p) * 128 + m) * NO + co];
+#pragma unroll 8
+        for (int b = b0; b < b1; ++b) s += src[b * stride];
+        s_part[w][lane] = s;
+    }
+    __syncthreads();
+    if (w == 0 && i < n) {
+        float s = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) s += s_part[q][lane];
         grads[i] = s;
     }
 }
@@ -688,22 +705,19 @@ mpm_status conv(mpm_ctx *ctx, mpm_cnn *c, tc::ConvArgs A, int slot, cudaStream_t
     return MPM_OK;
 }
 
-template <int CI, int NO>
-mpm_status wgrad(mpm_ctx *ctx, mpm_cnn *c, const __nv_bfloat16 *in, const __nv_bfloat16 *g, int gc, int l,
-                 cudaStream_t st)
+template <int CI, int NO, int GC>
+mpm_status wgrad(mpm_ctx *ctx, mpm_cnn *c, const __nv_bfloat16 *in, const __nv_bfloat16 *g, int l, cudaStream_t st)
 {
     static bool attr = false;
     constexpr int smem = tc::WgSmem<CI, NO>::BYTES;
     if (!attr) {
-        cudaFuncSetAttribute(tc::k_wgrad_tc<CI, NO>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaFuncSetAttribute(tc::k_wgrad_tc<CI, NO, GC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         attr = true;
     }
     tc::WgradArgs A;
     memset(&A, 0, sizeof(A));
     A.in = in;
     A.g = g;
-    A.gc = gc;
-    A.mask = c->mask;
     A.dom = c->dom;
     A.units = c->units;
     A.nunits = c->counters;
@@ -712,8 +726,10 @@ mpm_status wgrad(mpm_ctx *ctx, mpm_cnn *c, const __nv_bfloat16 *in, const __nv_b
     A.partials = c->partials;
     A.err = c->d_err;
     A.timeout_ns = ctx->timeout_ns;
-    tc::k_wgrad_tc<CI, NO><<<ctx->num_sms, tc::kThreads, smem, st>>>(A);
-    k_wgrad_reduce<<<64, 256, 0, st>>>(c->partials, ctx->num_sms, CI, NO, chan(l), chan(l + 1), c->grads + c->off[l]);
+    tc::k_wgrad_tc<CI, NO, GC><<<ctx->num_sms, tc::kWgThreads, smem, st>>>(A);
+    const int n = 27 * chan(l) * chan(l + 1) + chan(l + 1);
+    k_wgrad_reduce<<<(n + 31) / 32, 256, 0, st>>>(c->partials, ctx->num_sms, CI, NO, chan(l), chan(l + 1),
+                                                  c->grads + c->off[l]);
     ctx->launches += 2;
     return mpm_cuda_check(ctx, cudaGetLastError(), "cnn weight gradient");
 }
@@ -1098,9 +1114,9 @@ extern "C" mpm_status mpm_cnn_train_step(mpm_ctx *ctx, mpm_cnn *c, int32_t nimg,
     for (int l = kLayers - 1; l >= 0; --l) {
         const __nv_bfloat16 *in = l == 0 ? c->x : c->a[l - 1];
         const __nv_bfloat16 *gl = l == kLayers - 1 ? c->g6 : g;
-        if (l == kLayers - 1) r = wgrad<kHC, 16>(ctx, c, in, gl, kGC6, l, st);
-        else if (l == 0) r = wgrad<kXC, 32>(ctx, c, in, gl, kHC, l, st);
-        else r = wgrad<kHC, 32>(ctx, c, in, gl, kHC, l, st);
+        if (l == kLayers - 1) r = wgrad<kHC, 16, kGC6>(ctx, c, in, gl, l, st);
+        else if (l == 0) r = wgrad<kXC, 32, kHC>(ctx, c, in, gl, l, st);
+        else r = wgrad<kHC, 32, kHC>(ctx, c, in, gl, l, st);
         if (r != MPM_OK) return r;
         if (l == 0) break;
         tc::ConvArgs A;

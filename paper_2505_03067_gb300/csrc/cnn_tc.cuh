@@ -31,15 +31,15 @@
 // slots; one warp issues each depth's MMAs (the tap depths folded into N)
 // into the accumulators of the slabs it feeds and commits them to
 // mbarriers; epilogue warps drain complete slabs (tcgen05.ld) while the
-// tensor cores run on.  The weight-gradient kernel runs its own, simpler
-// pipeline (kSlots slots, eight warps).
+// tensor cores run on.  The weight-gradient kernel has loader warps and an MMA
+// warp of the same kind; its accumulators are read out once, at its end.
 //
 // Weight gradient.  dW[(dx,dy,dz)][ci][co] = sum_v in[v + off][ci] g[v][co] is
 // a GEMM over voxels with the halo buffer read as an MN-major A operand
 // (M = the K-columns of the forward layout, K = voxels along y) and the
-// slab's gradient tile as an MN-major B operand; the nine taps accumulate in
-// nine TMEM accumulators over all slabs of a CTA, and per-CTA partial sums are
-// reduced in a fixed order.
+// slabs' gradient tiles as an MN-major B operand, the tap depths folded into N;
+// the nine tap pairs accumulate in TMEM over all slabs of a CTA, and per-CTA
+// partial sums are reduced in a fixed order.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -51,8 +51,6 @@ namespace tc {
 
 constexpr int kSlabX = 8, kSlabY = 16, kZSeg = 8;
 constexpr int kHaloX = kSlabX + 2, kHaloY = kSlabY + 2;
-constexpr int kSlots = 6;               // halo depths in the shared-memory ring
-constexpr int kThreads = 256;           // weight-gradient kernel: 8 warps
 // forward kernel: 12 epilogue warps, 6 loader warps and one warp that issues the
 // MMAs (19 warps, at most 5 on each SM sub-partition; 96 registers a thread).
 // With six loader warps a thread issues 7 halo copies per depth instead of
@@ -91,14 +89,6 @@ struct Unit {
 // ---------------------------------------------------------------- PTX helpers
 __device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
-// Shared-memory matrix descriptor, no swizzle: start address, K-direction
-// core-matrix stride (LBO) and M/N-direction stride (SBO), sm_100 version bit.
-__device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t sbo)
-{
-    return (uint64_t)((addr & 0x3FFFFu) >> 4) | ((uint64_t)((lbo >> 4) & 0x3FFFu) << 16) |
-           ((uint64_t)((sbo >> 4) & 0x3FFFu) << 32) | (1ull << 46);
-}
-
 // Instruction descriptor of kind::f16 with bf16 A and B, FP32 accumulation.
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool b_mn)
 {
@@ -106,14 +96,7 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool a_mn, bool 
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum)
-{
-    asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(d_tmem),
-                 "l"(a), "l"(b), "r"(idesc), "r"(accum));
-}
-
-// The same issued by a converged warp: every lane executes it with the same
+// One MMA issued by a converged warp: every lane executes it with the same
 // (warp-uniform) operands and one elected lane issues.  Descriptors come as
 // their two 32-bit words (the start address and LBO in the low word), so a
 // tile offset is one 32-bit add.
@@ -133,18 +116,14 @@ __device__ __forceinline__ void mma_commit_warp(uint64_t *bar)
                  : "memory");
 }
 
-// Low and high words of a no-swizzle shared-memory descriptor (see sdesc).
+// Low and high words of a shared-memory matrix descriptor, no swizzle: start
+// address and K-direction core-matrix stride (LBO); M/N-direction stride
+// (SBO) and the sm_100 version bit.
 __device__ __forceinline__ uint32_t sdesc_lo(uint32_t addr, uint32_t lbo)
 {
     return ((addr & 0x3FFFFu) >> 4) | (((lbo >> 4) & 0x3FFFu) << 16);
 }
 __host__ __device__ constexpr uint32_t sdesc_hi(uint32_t sbo) { return ((sbo >> 4) & 0x3FFFu) | (1u << 14); }
-
-__device__ __forceinline__ void mma_commit(uint64_t *bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
 
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
 {
@@ -171,22 +150,6 @@ __device__ __forceinline__ bool mbar_try_sleep(uint64_t *bar, uint32_t parity, u
                  : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
                  : "memory");
     return ok != 0;
-}
-
-// Bounded wait for phase `parity` of an mbarrier: false (and *err set) when
-// timeout_ns of wall time passed.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, uint64_t timeout_ns, int32_t *err)
-{
-    if (mbar_try(bar, parity)) return true;
-    const uint64_t t0 = globaltimer_ns();
-    for (;;) {
-        for (int i = 0; i < 64; ++i)
-            if (mbar_try(bar, parity)) return true;
-        if (globaltimer_ns() - t0 > timeout_ns) {
-            if (err) atomicExch(err, 1);
-            return false;
-        }
-    }
 }
 
 __device__ __forceinline__ void tmem_alloc(uint32_t *slot, uint32_t ncols)
@@ -237,18 +200,6 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8])
     for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
-{
-    uint32_t r[16];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-                   "=r"(r[15])
-                 : "r"(taddr));
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 // 16-byte asynchronous global -> shared copy; src_bytes 0 writes zeros.  The
 // copy allocates in L1 (.ca): the three x-shifted halo copies read each
 // 16-byte source chunk three times, and the second and third reads hit L1.
@@ -256,19 +207,8 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-// Wait until at most n of this thread's committed groups are pending.
-__device__ __forceinline__ void cp_async_wait(int n)
-{
-    switch (n) {
-    case 0: asm volatile("cp.async.wait_group 0;" ::: "memory"); break;
-    case 1: asm volatile("cp.async.wait_group 1;" ::: "memory"); break;
-    case 2: asm volatile("cp.async.wait_group 2;" ::: "memory"); break;
-    case 3: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
-    case 4: asm volatile("cp.async.wait_group 4;" ::: "memory"); break;
-    default: asm volatile("cp.async.wait_group 5;" ::: "memory"); break;
-    }
-}
+// Wait for every copy this thread issued.
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // GELU(z) = z Phi(z), Phi(z) = (1 + erf(z / sqrt 2)) / 2, with erf from the
 // rational-exponential approximation of Abramowitz & Stegun, Handbook of
@@ -691,7 +631,7 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
             }
             if (s_lstop) break;
         }
-        cp_async_wait(0);
+        cp_async_wait_all();
     } else if (warp == kEpiWarps + kLoadWarps) {
         // ------------------------------------------------------------ MMA issue
         // The whole warp runs this loop on warp-uniform values (shared-memory
@@ -908,30 +848,40 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
 }
 
 // ---------------------------------------------------------------- weight gradient
+// Warps of the weight-gradient kernel: loaders, then the one that issues the
+// MMAs; all eight read the accumulators out at the end.
+constexpr int kWgLoadWarps = 6;
+constexpr int kWgThreads = 256;
+constexpr int kWgSlots = 6;             // halo depths in its ring
+constexpr int kWgTiles = 8;             // gradient tiles (output slabs) in theirs
+
 // Shared memory of the weight-gradient kernel: the halo ring (its pad column
 // q = QC holds ones, so the row block of that column accumulates the bias
-// gradient), a guard for the A operand's M overrun, two gradient tiles.
+// gradient), a guard for the A operand's M overrun, the ring of gradient
+// tiles [y][tile][channel group][x][8 channels], two units' activity bytes.
 template <int CI, int NO>
 struct WgSmem {
     static constexpr int NG = NO / 8;
     static constexpr int RING_OFF = 0;
-    static constexpr int RING_BYTES = kSlots * Halo<CI>::SLOT;
-    static constexpr int G_OFF = RING_OFF + RING_BYTES + 2048;
-    static constexpr int G_BYTES = kSlabY * NG * 128;
-    static constexpr int ACT_OFF = G_OFF + 2 * G_BYTES;
-    static constexpr int ACT_BYTES = kActStride;
-    static constexpr int BAR_OFF = (ACT_OFF + ACT_BYTES + 15) & ~15;
+    static constexpr int RING_BYTES = kWgSlots * Halo<CI>::SLOT;
+    static constexpr int G_OFF = (RING_OFF + RING_BYTES + 2048 + 1023) & ~1023;
+    static constexpr int YS = kWgTiles * NG * 128;                 // bytes per y
+    static constexpr int G_BYTES = kSlabY * YS;
+    static constexpr int ACT_OFF = G_OFF + G_BYTES;
+    // mbarriers: full[slots], empty[slots], all MMAs done
+    static constexpr int BAR_OFF = (ACT_OFF + 2 * kActStride + 15) & ~15;
+    static constexpr int NBAR = 2 * kWgSlots + 1;
     // more than half an SM's shared memory: one CTA per SM, so a CTA's TMEM
     // allocation never waits for another's
-    static constexpr int BYTES = BAR_OFF + 64 > 120 * 1024 ? BAR_OFF + 64 : 120 * 1024;
-    static constexpr int TMEM_COLS = 9 * NO <= 256 ? 256 : 512;
+    static constexpr int BYTES0 = BAR_OFF + NBAR * 8;
+    static constexpr int BYTES = BYTES0 > 120 * 1024 ? BYTES0 : 120 * 1024;
+    static constexpr int COLS = 9 * NO;
+    static constexpr int TMEM_COLS = COLS <= 256 ? 256 : 512;
 };
 
 struct WgradArgs {
     const __nv_bfloat16 *in;        // [B * V][CI] layer input
     const __nv_bfloat16 *g;         // [B * V][GC] dLoss/dz of the layer output
-    int32_t gc;                     // channels stored per voxel in g (8 or 24)
-    const uint8_t *mask;
     const CnnDom *dom;
     const Unit *units;
     const int32_t *nunits;
@@ -944,136 +894,190 @@ struct WgradArgs {
 
 // Per CTA, over the units i = blockIdx, blockIdx + gridDim, ... (a fixed
 // assignment, so the partial sums and their fixed-order reduction are
-// reproducible): D_p[m][n] += sum over the slab's voxels v of
-// halo_(dy,dz)[v][m] g[v][n] for the nine tap pairs p = (dy, dz), m the row
-// (dx copy, channel) of the forward layout's K-columns.
-template <int CI, int NO>
-__global__ void __launch_bounds__(kThreads, 1) k_wgrad_tc(const __grid_constant__ WgradArgs A)
+// reproducible): D_(dy,dz)[m][n] += sum over the slabs' voxels v of
+// in[v + (dy, dz)][m] g[v][n], m the row (dx copy, channel) of the forward
+// layout's K-columns.  Both operands are MN-major (K = the voxels of two y
+// rows).
+//
+// As in the forward kernel the MMAs run depth by depth and the tap depths are
+// folded into N: input depth j meets the gradient tiles of slabs j - 2, j - 1
+// and j (dz = +1, 0, -1), which lie side by side along N in the tile ring (a
+// window that crosses the ring's end is issued in two parts), and their
+// accumulators lie side by side in TMEM: column block 3 (dy + 1) + 1 - dz.  An
+// MMA costs its operands' reads from shared memory, nearly independent of N
+// (46 cycles at N = 32, 56 at 96), so 24 MMAs a depth replace 72 a slab.
+// Six loader warps copy the halo depths and gradient tiles (cp.async, zeros
+// at inactive voxels) ahead of the warp that issues the MMAs.  A ring slot is
+// refilled once the MMAs of the depth that used it are complete; a gradient
+// tile's last use (two depths after its own, in another unit than the slab
+// that replaces it) is then complete as well, as kWgSlots <= 8.
+// GC: channels stored per voxel in g.  24 -> 24 channels on 8 images of 32^3:
+// 90 us with one MMA per tap pair and slab, one thread issuing them between
+// CTA-wide barriers; 32 us now.
+template <int CI, int NO, int GC>
+__global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ WgradArgs A)
 {
     using H = Halo<CI>;
     using S = WgSmem<CI, NO>;
+    constexpr int NLD = 32 * kWgLoadWarps;
+    constexpr int GCH = GC / 8;
+    constexpr int GI = (kSlabY * kSlabX * GCH + NLD - 1) / NLD;   // gradient copies per loader and tile
+    static_assert(kWgSlots <= 8 && kWgTiles == kZSeg && GCH <= S::NG, "tile ring");
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ uint32_t s_tmem;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(sm + S::BAR_OFF);
-    uint8_t *act = sm + S::ACT_OFF;
+    __shared__ int32_t s_abort;
+    __shared__ volatile int32_t s_lstop[2];       // by the depth's parity: read before it is written again
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + S::BAR_OFF), *empty = full + kWgSlots, *done = empty + kWgSlots;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const CnnDom &D = *A.dom;
     const uint32_t rbase = smem_u32(sm + S::RING_OFF), gbase = smem_u32(sm + S::G_OFF);
+    volatile int32_t *abort = &s_abort;
+    const uint64_t T = A.timeout_ns;
 
     // ring: zeros, ones in the pad column q = QC (CI = 24); gradient tiles: zeros
-    for (int i = tid; i < (S::RING_BYTES + 2048) / 16; i += kThreads) {
+    for (int i = tid; i < (S::RING_BYTES + 2048) / 16; i += kWgThreads) {
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
         const int off = i * 16;
         if (H::QP > H::QC && off < S::RING_BYTES && ((off % H::GS) / 128) == H::QC)
             w = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);   // bf16 1.0
         reinterpret_cast<uint4 *>(sm + S::RING_OFF)[i] = w;
     }
-    for (int i = tid; i < 2 * S::G_BYTES / 16; i += kThreads)
+    for (int i = tid; i < S::G_BYTES / 16; i += kWgThreads)
         reinterpret_cast<uint4 *>(sm + S::G_OFF)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (warp == 0) tmem_alloc(&s_tmem, S::TMEM_COLS);
     if (tid == 0) {
-        mbar_init(&bars[0], 1);
-        mbar_init(&bars[1], 1);
+        s_abort = 0;
+        for (int i = 0; i < kWgSlots; ++i) {
+            mbar_init(&full[i], NLD);
+            mbar_init(&empty[i], 1);
+        }
+        mbar_init(done, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     fence_async_smem();
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
     const uint32_t tmem = s_tmem;
-    constexpr uint32_t kIdesc = idesc_bf16(128, NO, true, true);
-    uint32_t nmma = 0;
-    bool ok = true;
-    const int nunits = *A.nunits;
-    HaloItems<CI, kThreads> items;
-    items.init(tid, D.L[0]);
-    const int gch = A.gc / 8;                     // real 8-channel chunks of g
-    for (int ui = blockIdx.x; ui < nunits && ok; ui += gridDim.x) {
-        const Unit u = A.units[ui];
-        copy_unit_act<kThreads>(A.uact, ui, act, tid);
-        __syncthreads();
-        const uint32_t bits = A.ubits[ui];
-        const int ndep = u.nz + 2;
-        int issued = 0;
-        for (; issued < ndep && issued < kSlots; ++issued) {
-            load_halo_depth_items<CI, kThreads>(D, A.in, u, act, issued, rbase + (issued % kSlots) * H::SLOT, items);
-            cp_async_commit();
-        }
-        for (int k = 0; k < u.nz && ok; ++k) {
-            if ((bits >> k) & 1u) {
-                const uint32_t m = nmma, buf = m & 1u;
-                // the gradient tile buffer was last read by MMA group m - 2
-                if (m >= 2 && tid == 0) ok = mbar_wait(&bars[buf], ((m - 2) >> 1) & 1u, A.timeout_ns, A.err);
-                ok = __syncthreads_and(ok);
-                if (!ok) break;
-                // gradient tile of slab k: [y][ng][x][8 channels], zero where inactive
-                unsigned char *gt = sm + S::G_OFF + buf * S::G_BYTES;
-                for (int i = tid; i < kSlabY * kSlabX * gch; i += kThreads) {
-                    const int ch = i % gch, r = i / gch;
-                    const int x = r % kSlabX, y = r / kSlabX;
-                    uint4 w = make_uint4(0u, 0u, 0u, 0u);
-                    if (act[((k + 1) * kHaloY + y + 1) * kHaloX + x + 1])
-                        w = __ldg(reinterpret_cast<const uint4 *>(
-                            A.g + vox_index(D, u.b, u.ox + x, u.oy + y, u.z0 + k) * A.gc + ch * 8));
-                    *reinterpret_cast<uint4 *>(gt + (y * S::NG + ch) * 128 + x * 16) = w;
-                }
-                cp_async_wait(issued - (k + 3) < 0 ? 0 : issued - (k + 3));
-                fence_async_smem();
-                tc_before_sync();
-                __syncthreads();
-                tc_after_sync();
-                if (tid == 0) {
-                    const uint32_t gb = gbase + buf * S::G_BYTES;
-#pragma unroll 1
-                    for (int p = 0; p < 9; ++p) {
-                        const int dy = p % 3 - 1, dz = p / 3 - 1;
-                        const uint32_t slot = (uint32_t)((k + 1 + dz) % kSlots);
-                        const uint32_t a0 = rbase + slot * H::SLOT + (uint32_t)(dy + 1) * H::GS;
-#pragma unroll
-                        for (int s = 0; s < kSlabY / 2; ++s) {
-                            const uint64_t ad = sdesc(a0 + 2u * s * H::GS, H::GS, 128u);
-                            const uint64_t bd = sdesc(gb + 2u * s * S::NG * 128u, S::NG * 128u, 128u);
-                            mma_bf16(tmem + (uint32_t)(p * NO), ad, bd, kIdesc, (m > 0 || s > 0) ? 1u : 0u);
-                        }
-                    }
-                    mma_commit(&bars[buf]);
-                }
-                nmma = m + 1;
-                // every MMA of slabs < k is complete once group m - 1 is: the
-                // ring slot of depth k - 1 may then be refilled
-                if (m >= 1 && tid == 0) ok = mbar_wait(&bars[(m - 1) & 1u], ((m - 1) >> 1) & 1u, A.timeout_ns, A.err);
-                ok = __syncthreads_and(ok);
-            } else if (nmma >= 1) {
-                if (tid == 0) ok = mbar_wait(&bars[(nmma - 1) & 1u], ((nmma - 1) >> 1) & 1u, A.timeout_ns, A.err);
-                ok = __syncthreads_and(ok);
-            }
-            if (ok && k >= 1 && issued < ndep && issued == k - 1 + kSlots) {
-                load_halo_depth_items<CI, kThreads>(D, A.in, u, act, issued, rbase + (issued % kSlots) * H::SLOT, items);
-                cp_async_commit();
-                ++issued;
-            }
-        }
-        cp_async_wait(0);
-        __syncthreads();
+    if (warp < 4) {   // every accumulator starts at zero: the MMAs always accumulate
+        for (uint32_t c = 0; c < (uint32_t)S::COLS; c += 8) tmem_zero8(tmem + c + ((uint32_t)(warp * 32) << 16));
+        tc_wait_st();
     }
-    // the last group, then the accumulators to this CTA's partial sums
-    if (ok && nmma >= 1 && tid == 0) ok = mbar_wait(&bars[(nmma - 1) & 1u], ((nmma - 1) >> 1) & 1u, A.timeout_ns, A.err);
-    ok = __syncthreads_and(ok);
+    tc_before_sync();
+    __syncthreads();
     tc_after_sync();
+    const int nunits = *A.nunits;
+
+    if (warp < kWgLoadWarps) {
+        // ------------------------------------------------------------ loaders
+        HaloItems<CI, NLD> items;
+        items.init(tid, D.L[0]);
+        uint32_t dseq = 0, tseq = 0;              // depths, tiles issued
+        bool stop = false;
+        for (int ui = blockIdx.x, n = 0; ui < nunits && !stop; ui += gridDim.x, ++n) {
+            const Unit u = A.units[ui];
+            uint8_t *act = sm + S::ACT_OFF + (n & 1) * kActStride;   // its readers of two units ago passed a barrier since
+            copy_unit_act<NLD>(A.uact, ui, act, tid);
+            for (int j = 0; j < u.nz + 2; ++j) {
+                const uint32_t slot = dseq % kWgSlots, use = dseq / kWgSlots;
+                if (tid == 0)
+                    s_lstop[dseq & 1] = use >= 1 && !mbar_wait_or_abort(&empty[slot], (use - 1) & 1, T, A.err, abort);
+                named_sync(1, NLD);
+                stop = s_lstop[dseq & 1] != 0;
+                if (stop) break;
+                load_halo_depth_items<CI, NLD>(D, A.in, u, act, j, rbase + slot * H::SLOT, items);
+                if (j < u.nz) {                   // the gradient tile of slab j
+                    const int64_t v0 = vox_index(D, u.b, u.ox, u.oy, u.z0 + j);
+                    const uint32_t dst = gbase + (tseq % kWgTiles) * (S::NG * 128);
+#pragma unroll
+                    for (int k = 0; k < GI; ++k) {
+                        const int i = tid + k * NLD;
+                        if (i >= kSlabY * kSlabX * GCH) continue;
+                        const int x = i % kSlabX, r = i / kSlabX;   // x fastest: a core matrix's 128 bytes together
+                        const int ch = r % GCH, y = r / GCH;
+                        const bool on = act[((j + 1) * kHaloY + y + 1) * kHaloX + x + 1] != 0;
+                        const __nv_bfloat16 *src = on ? A.g + (v0 + (int64_t)y * D.L[0] + x) * GC + ch * 8 : A.g;
+                        cp_async16(dst + (uint32_t)(y * S::YS + ch * 128 + x * 16), src, on ? 16u : 0u);
+                    }
+                    ++tseq;
+                }
+                cp_async_arrive(&full[slot]);
+                ++dseq;
+            }
+        }
+        cp_async_wait_all();
+    } else if (warp == kWgLoadWarps) {
+        // ------------------------------------------------------------ MMA issue
+        // warp-uniform operands, one elected lane issuing (see k_conv_tc)
+        constexpr uint32_t kId[4] = {0u, idesc_bf16(128, NO, true, true), idesc_bf16(128, 2 * NO, true, true),
+                                     idesc_bf16(128, 3 * NO, true, true)};
+        const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
+        const uint32_t alo0 = sdesc_lo(rbase, H::GS), blo0 = sdesc_lo(gbase, S::YS);
+        constexpr uint32_t ahi = sdesc_hi(128u), bhi = sdesc_hi(128u);
+        uint32_t d = 0, t0 = 0;
+        bool ok = true;
+        for (int ui = blockIdx.x; ui < nunits && ok; ui += gridDim.x) {
+            const int nz = __shfl_sync(0xffffffffu, A.units[ui].nz, 0);
+            const uint32_t bits = __shfl_sync(0xffffffffu, A.ubits[ui], 0) & ((1u << nz) - 1u);
+            for (int j = 0; j < nz + 2; ++j, ++d) {
+                const uint32_t slot = d % kWgSlots;
+                ok = mbar_wait_warp(&full[slot], (d / kWgSlots) & 1, T, A.err, abort);
+                if (!ok) break;
+                fence_async_smem();
+                tc_after_sync();
+                // slabs klo .. khi of the window that are active, as one or two runs of ring tiles
+                const int k0 = j >= 2 ? j - 2 : 0, k1 = j < nz ? j : nz - 1;
+                const uint32_t sel = (bits >> k0) & ((2u << (k1 - k0)) - 1u);
+                if (sel) {
+                    int k = k0 + __ffs(sel) - 1;
+                    const int khi = k0 + 31 - __clz(sel);
+                    while (k <= khi) {
+                        const uint32_t tile = (t0 + (uint32_t)k) % kWgTiles;
+                        const int run = min(khi - k + 1, (int)(kWgTiles - tile));
+                        const uint32_t idn = run == 3 ? kId[3] : (run == 2 ? kId[2] : kId[1]);
+                        // column block of dz = j - 1 - k: 1 - dz = k - j + 2
+                        const uint32_t dacc = tm + (uint32_t)(NO * (k - j + 2));
+                        const uint32_t alo = alo0 + slot * (uint32_t)(H::SLOT >> 4);
+                        const uint32_t blo = blo0 + tile * (uint32_t)(S::NG * 8);
+#pragma unroll
+                        for (int i = 0; i < 3 * (kSlabY / 2); ++i) {
+                            const int dyi = i / (kSlabY / 2), s2 = i % (kSlabY / 2);
+                            mma_bf16_warp(dacc + (uint32_t)(3 * NO * dyi),
+                                          alo + (uint32_t)(((dyi + 2 * s2) * H::GS) >> 4), ahi,
+                                          blo + (uint32_t)((2 * s2 * S::YS) >> 4), bhi, idn, 1u);
+                        }
+                        k += run;
+                    }
+                }
+                mma_commit_warp(&empty[slot]);
+            }
+            t0 += (uint32_t)nz;
+        }
+        mma_commit_warp(done);
+        if (ok) ok = mbar_wait_warp(done, 0, T, A.err, abort);
+        __syncwarp();
+    }
+    // every role is done (or gave up): the accumulators to this CTA's partial sums
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    const bool zero = s_abort != 0;
     const int lq = warp & 3, half = warp >> 2;
     const int row = lq * 32 + lane;
-    if (half * 16 < NO) {
-        for (int p = 0; p < 9; ++p) {
-            float v[16];
-            tmem_ld16(tmem + (uint32_t)(p * NO + half * 16) + ((uint32_t)(lq * 32) << 16), v);
-            tc_wait_ld();
-            float4 *o = reinterpret_cast<float4 *>(A.partials + (((size_t)blockIdx.x * 9 + p) * 128 + row) * NO + half * 16);
-            const bool z = nmma == 0 || !ok;
+    if (lq * 32 < H::QP * 8) {                    // rows past the K-columns are never read
+        for (int pb = half; pb < 9; pb += 2) {    // column block pb: dy = pb / 3 - 1, dz = 1 - pb % 3
+            const int p = pb / 3 + 3 * (2 - pb % 3);
+            float4 *o = reinterpret_cast<float4 *>(A.partials + (((size_t)blockIdx.x * 9 + p) * 128 + row) * NO);
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
-                o[i] = z ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            for (int cg = 0; cg < GCH; ++cg) {
+                float v[8];
+                tmem_ld8(tmem + (uint32_t)(pb * NO + cg * 8) + ((uint32_t)(lq * 32) << 16), v);
+                tc_wait_ld();
+                o[2 * cg] = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(v[0], v[1], v[2], v[3]);
+                o[2 * cg + 1] = zero ? make_float4(0.f, 0.f, 0.f, 0.f) : make_float4(v[4], v[5], v[6], v[7]);
+            }
         }
     }
-    cp_async_wait(0);
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
