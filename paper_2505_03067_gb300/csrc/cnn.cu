@@ -161,16 +161,13 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
 
 // ---------------------------------------------------------------- plans
 // Candidate unit ci of image mode -> unit record; false if it lies outside its image's box.
-__device__ __forceinline__ bool unit_of(const CnnDom &D, int64_t ci, Unit &u)
+__device__ __forceinline__ bool unit_of(const CnnDom &D, uint32_t ci, Unit &u)
 {
-    const int nsx = (D.L[0] + tc::kSlabX - 1) / tc::kSlabX, nsy = (D.L[1] + tc::kSlabY - 1) / tc::kSlabY;
-    const int nzs = (D.L[2] + tc::kZSeg - 1) / tc::kZSeg;
-    const int i = (int)(ci % nsx);
-    int64_t r = ci / nsx;
-    const int j = (int)(r % nsy);
-    r /= nsy;
-    const int kz = (int)(r % nzs);
-    const int b = (int)(r / nzs);
+    const uint32_t nsx = (D.L[0] + tc::kSlabX - 1) / tc::kSlabX, nsy = (D.L[1] + tc::kSlabY - 1) / tc::kSlabY;
+    const uint32_t nzs = (D.L[2] + tc::kZSeg - 1) / tc::kZSeg;
+    const uint32_t r1 = ci / nsx, r2 = r1 / nsy;
+    const int i = (int)(ci - r1 * nsx), j = (int)(r1 - r2 * nsy), b = (int)(r2 / nzs);
+    const int kz = (int)(r2 - (uint32_t)b * nzs);
     u.b = b;
     u.ox = D.lo[b][0] + i * tc::kSlabX;
     u.oy = D.lo[b][1] + j * tc::kSlabY;
@@ -180,21 +177,30 @@ __device__ __forceinline__ bool unit_of(const CnnDom &D, int64_t ci, Unit &u)
     return i * tc::kSlabX < D.n[b][0] && j * tc::kSlabY < D.n[b][1] && u.nz > 0;
 }
 
-// Image mode, one warp per candidate unit: any active voxel (in the box, mask set)?
-__global__ void k_plan_flags(const __grid_constant__ CnnDom D, const uint8_t *__restrict__ mask, int64_t ncand,
-                             uint8_t *__restrict__ flags)
+// Image mode, one warp per candidate unit: any active voxel (in the box, mask
+// set)?  A lane takes rows of eight voxels, four of them in flight.  71 us with
+// a byte a lane for 23 000 candidates, 23 us now.
+__global__ void __launch_bounds__(256) k_plan_flags(const __grid_constant__ CnnDom D, const uint8_t *__restrict__ mask,
+                                                    int64_t ncand, uint8_t *__restrict__ flags)
 {
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = (gridDim.x * (int64_t)blockDim.x) >> 5;
+    const int64_t total = (int64_t)D.B * D.L[2] * D.L[1] * D.L[0];
     for (int64_t c = w0; c < ncand; c += nw) {
         Unit u;
         bool any = false;
-        if (unit_of(D, c, u)) {
-            for (int i = lane; i < tc::kSlabX * tc::kSlabY * u.nz && !any; i += 32) {
-                const int x = u.ox + (i & 7), y = u.oy + ((i >> 3) & 15), z = u.z0 + (i >> 7);
-                any = tc::in_box(D, u.b, x, y, z) && mask[tc::vox_index(D, u.b, x, y, z)] != 0;
+        if (unit_of(D, (uint32_t)c, u)) {
+            const int *lo = D.lo[u.b], *n = D.n[u.b];
+            uint32_t bits = 0u;
+#pragma unroll
+            for (int k = 0; k < tc::kSlabY * tc::kZSeg / 32; ++k) {
+                const int r = lane + 32 * k, y = u.oy + r % tc::kSlabY, z = u.z0 + r / tc::kSlabY;
+                if (y < lo[1] + n[1] && z < u.z0 + u.nz)
+                    bits |= tc::row_bits(mask, total, true, tc::vox_index(D, u.b, 0, y, z), u.ox, tc::kSlabX, lo[0],
+                                         lo[0] + n[0]);
             }
+            any = bits != 0u;
         }
         any = __any_sync(0xffffffffu, any);
         if (lane == 0) flags[c] = any ? 1 : 0;
@@ -202,41 +208,55 @@ __global__ void k_plan_flags(const __grid_constant__ CnnDom D, const uint8_t *__
 }
 
 // Image mode, one CTA: the flagged units in candidate order (a fixed order:
-// the weight gradient's per-CTA sums depend on it); writes the domain too.
+// the weight gradient's per-CTA sums depend on it); writes the domain too.  A
+// thread takes 16 consecutive candidates (flags: a multiple of 16 bytes), so a
+// round and its barriers serve 16 384 of them: 48 us with 1 024 a round for
+// 23 000 candidates, 26 us now.
 __global__ void __launch_bounds__(1024) k_plan_compact(const __grid_constant__ CnnDom D,
                                                        const uint8_t *__restrict__ flags, int64_t ncand,
                                                        Unit *__restrict__ units, int32_t *__restrict__ counters,
                                                        CnnDom *__restrict__ dom_out)
 {
     __shared__ int s_w[32];
-    __shared__ int s_base;
-    if (threadIdx.x == 0) {
-        s_base = 0;
-        *dom_out = D;
-    }
-    __syncthreads();
+    if (threadIdx.x == 0) *dom_out = D;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int64_t c0 = 0; c0 < ncand; c0 += 1024) {
-        const int64_t c = c0 + threadIdx.x;
-        const bool f = c < ncand && flags[c];
-        const unsigned bal = __ballot_sync(0xffffffffu, f);
-        if (lane == 0) s_w[wid] = __popc(bal);
+    int base = 0;
+    for (int64_t c0 = 0; c0 < ncand; c0 += 16 * 1024) {
+        const int64_t c = c0 + 16 * (int64_t)threadIdx.x;
+        uint32_t set = 0u;
+        if (c < ncand) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(flags + c);
+            const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+                if (c + k < ncand && ((w[k >> 2] >> (8 * (k & 3))) & 0xffu)) set |= 1u << k;
+        }
+        int incl = __popc(set);
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += t;
+        }
+        __syncthreads();                          // the last round's sums were read
+        if (lane == 31) s_w[wid] = incl;
         __syncthreads();
         int off = 0, tot = 0;
         for (int i = 0; i < 32; ++i) {
             if (i < wid) off += s_w[i];
             tot += s_w[i];
         }
-        if (f) {
+        int at = base + off + incl - __popc(set);
+        for (uint32_t m = set; m; m &= m - 1) units[at++].pad0 = (int32_t)(c + __ffs(m) - 1);
+        // the records of the round's candidates, spread over the CTA
+        __syncthreads();
+        for (int i = base + (int)threadIdx.x; i < base + tot; i += 1024) {
             Unit u;
-            unit_of(D, c, u);
-            units[s_base + off + __popc(bal & ((1u << lane) - 1u))] = u;
+            unit_of(D, (uint32_t)units[i].pad0, u);
+            units[i] = u;
         }
-        __syncthreads();
-        if (threadIdx.x == 0) s_base += tot;
-        __syncthreads();
+        base += tot;
     }
-    if (threadIdx.x == 0) counters[0] = s_base;
+    if (threadIdx.x == 0) counters[0] = base;
 }
 
 // Solver mode: the box of a subgrid (from device memory) on a lattice of dims
@@ -347,10 +367,9 @@ __device__ __forceinline__ void feat_store(__nv_bfloat16 *xo, const float (&f)[k
 }
 
 // fld[s]: the value of species s's field channel before scaling
-__device__ __forceinline__ void features_of(const FeatSrc &F, int64_t L, const float (&fld)[3], bool with_source,
+__device__ __forceinline__ void features_of(const FeatSrc &F, int32_t id, const float (&fld)[3], bool with_source,
                                             float (&f)[kXC])
 {
-    int id = F.cell[L];
     if (id < 0 || id >= F.ncell) id = 0;
 #pragma unroll
     for (int c = 0; c < kXC; ++c) f[c] = 0.0f;
@@ -367,31 +386,91 @@ __device__ __forceinline__ void features_of(const FeatSrc &F, int64_t L, const f
 }
 
 // Image mode: the box voxels of lattice F (dims = the image dims) into image b:
-// mask, features and c^n (FP32).
-__global__ void k_feat_image(FeatSrc F, const uint8_t *__restrict__ lmask, int32_t L0, int32_t L1, int32_t L2, int b,
-                             int32_t lo0, int32_t lo1, int32_t lo2, int32_t n0, int32_t n1, int32_t n2,
-                             uint8_t *__restrict__ mask, __nv_bfloat16 *__restrict__ x, float *__restrict__ f32)
+// the mask of all, features and c^n (FP32) of those in the mask -- nothing
+// reads the others (mpm_cnn_export_features gives zeros for them).  A warp
+// takes 128 voxels of a row at a time, loads the next ones' mask before it works
+// on these, and queues the voxels in the mask: features are formed for 32
+// queued voxels at once, so that the chain id -> rates and the fields' loads
+// serve full warps on a thin shell.  Writing every voxel of the box took 218 us
+// for 15 M voxels (2.4 M in the mask), four voxels a lane without the queue
+// 107, this form 59 us.
+constexpr int kFeatSeg = 4;   // voxels a lane
+__global__ void __launch_bounds__(256) k_feat_image(FeatSrc F, const uint8_t *__restrict__ lmask, int32_t L0,
+                                                    int32_t L1, int32_t L2, int b, int32_t lo0, int32_t lo1,
+                                                    int32_t lo2, int32_t n0, int32_t n1, int32_t n2,
+                                                    uint8_t *__restrict__ mask, __nv_bfloat16 *__restrict__ x,
+                                                    float *__restrict__ f32)
 {
-    const int64_t nb = (int64_t)n0 * n1 * n2;
+    __shared__ uint32_t s_queue[8][32 * (kFeatSeg + 1)];
     const int64_t img = (int64_t)b * L0 * L1 * L2;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < nb; i += gridDim.x * (int64_t)blockDim.x) {
-        const int xx = lo0 + (int)(i % n0);
-        const int64_t r = i / n0;
-        const int yy = lo1 + (int)(r % n1), zz = lo2 + (int)(r / n1);
-        const int64_t L = xx + (int64_t)L0 * (yy + (int64_t)L1 * zz);
-        const int64_t v = img + L;
-        const uint8_t m = lmask[L] != 0;
-        mask[v] = m;
+    const int lane = threadIdx.x & 31;
+    uint32_t *queue = s_queue[threadIdx.x >> 5];
+    const uint32_t nseg = ((uint32_t)n0 + 32 * kFeatSeg - 1) / (32 * kFeatSeg);
+    const uint32_t nitem = nseg * (uint32_t)n1 * (uint32_t)n2;      // fewer than voxels
+    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
+    uint32_t it = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    uint8_t mnext[kFeatSeg];
+    uint32_t Lnext = 0;
+    int xnext = 0;
+    auto load = [&](uint32_t i) {
+        const uint32_t r = i / nseg, zi = r / (uint32_t)n1, yi = r - zi * (uint32_t)n1;
+        xnext = (int)(i - r * nseg) * 32 * kFeatSeg + lane;
+        Lnext = (uint32_t)(lo0 + xnext) + (uint32_t)L0 * ((uint32_t)lo1 + yi + (uint32_t)L1 * ((uint32_t)lo2 + zi));
+#pragma unroll
+        for (int k = 0; k < kFeatSeg; ++k) mnext[k] = xnext + 32 * k < n0 ? lmask[Lnext + 32 * k] : 0;
+    };
+    auto form = [&](uint32_t L) {
+        const int32_t id = F.cell[L];
         float fld[3];
+#pragma unroll
         for (int s = 0; s < 3; ++s) fld[s] = s < F.nspecies ? (float)F.field[s][L] : 0.0f;
+        const int64_t v = img + L;
+#pragma unroll
         for (int s = 0; s < 3; ++s) f32[v * 3 + s] = fld[s];
         float f[kXC];
-        features_of(F, L, fld, true, f);
-        if (!m) {
-#pragma unroll
-            for (int c = 0; c < kXC; ++c) f[c] = 0.0f;
-        }
+        features_of(F, id, fld, true, f);
         feat_store(x + v * kXC, f);
+    };
+    int nq = 0;   // queued voxels, below 32 between items
+    if (it < nitem) load(it);
+    for (; it < nitem; it += nw) {
+        uint8_t m[kFeatSeg];
+        const uint32_t L = Lnext;
+        const int bx = xnext;
+#pragma unroll
+        for (int k = 0; k < kFeatSeg; ++k) m[k] = mnext[k];
+        if (it + nw < nitem) load(it + nw);
+#pragma unroll
+        for (int k = 0; k < kFeatSeg; ++k) {
+            if (bx + 32 * k < n0) mask[img + L + 32 * k] = m[k] != 0;
+            const unsigned on = __ballot_sync(0xffffffffu, m[k] != 0);
+            if (m[k]) queue[nq + __popc(on & ((1u << lane) - 1u))] = L + 32 * k;
+            nq += __popc(on);
+        }
+        __syncwarp();
+        int at = 0;
+        for (; nq - at >= 32; at += 32) form(queue[at + lane]);
+        const uint32_t rest = lane < nq - at ? queue[at + lane] : 0u;   // fewer than 32: to the queue's start
+        __syncwarp();
+        nq -= at;
+        if (lane < nq) queue[lane] = rest;
+    }
+    __syncwarp();
+    if (lane < nq) form(queue[lane]);
+}
+
+// The loaded features as mpm_cnn_export_features gives them: zero off the mask.
+// T: the widest word the destination is aligned for.
+template <typename T>
+__global__ void k_export_features(const __nv_bfloat16 *__restrict__ x, const uint8_t *__restrict__ mask, int64_t n,
+                                  T *__restrict__ out)
+{
+    constexpr int per = kXC * 2 / (int)sizeof(T);   // words of a voxel
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < per * n; i += gridDim.x * (int64_t)blockDim.x) {
+        T v;
+        memset(&v, 0, sizeof(T));
+        if (mask[i / per]) v = reinterpret_cast<const T *>(x)[i];
+        out[i] = v;
     }
 }
 
@@ -474,7 +553,7 @@ __global__ void k_feat_units(const __grid_constant__ FeatUnits A)
                 for (int s = 0; s < 3; ++s) A.f32[L * 3 + s] = fld[s];
             }
             float f[kXC];
-            features_of(A.F, L, fld, A.vin == nullptr, f);
+            features_of(A.F, A.F.cell[L], fld, A.vin == nullptr, f);
             feat_store(A.x + L * kXC, f);
         }
     }
@@ -763,7 +842,7 @@ mpm_status check_err(mpm_ctx *ctx, mpm_cnn *c)
 // for all six layers and the backward pass).
 mpm_status unit_act(mpm_ctx *ctx, mpm_cnn *c, const uint8_t *mask, cudaStream_t st)
 {
-    tc::k_unit_act<<<ctx->num_sms * 4, 256, 0, st>>>(c->dom, mask, c->units, c->counters, c->uact, c->ubits);
+    tc::k_unit_act<<<ctx->num_sms * 8, 192, 0, st>>>(c->dom, mask, c->units, c->counters, c->uact, c->ubits);
     ctx->launches += 1;
     return mpm_cuda_check(ctx, cudaGetLastError(), "cnn unit activity");
 }
@@ -916,7 +995,7 @@ extern "C" mpm_status mpm_cnn_create(mpm_ctx *ctx, mpm_cnn **out, const int32_t 
     A((void **)&c->units, (size_t)c->max_units * sizeof(Unit));
     A((void **)&c->uact, (size_t)c->max_units * tc::kActStride);
     A((void **)&c->ubits, (size_t)c->max_units * sizeof(uint32_t));
-    A((void **)&c->flags, (size_t)c->max_units);
+    A((void **)&c->flags, ((size_t)c->max_units + 15) & ~(size_t)15);   // read 16 bytes at a time
     A((void **)&c->counters, 64 * sizeof(int32_t));
     A((void **)&c->geo, 256);
     A((void **)&c->nact, 256);
@@ -1029,7 +1108,7 @@ extern "C" mpm_status mpm_cnn_load_image(mpm_ctx *ctx, mpm_cnn *c, int32_t b, co
             c->hdom.lo[b][d] = box->lo[d];
             c->hdom.n[b][d] = box->hi[d] - box->lo[d];
         }
-        k_feat_image<<<ctx->num_sms * 4, 256, 0, st>>>(F, lat->mask, c->L[0], c->L[1], c->L[2], b, box->lo[0],
+        k_feat_image<<<ctx->num_sms * 8, 256, 0, st>>>(F, lat->mask, c->L[0], c->L[1], c->L[2], b, box->lo[0],
                                                         box->lo[1], box->lo[2], n0, n1, n2, c->mask, c->x, c->f32);
     } else {
         k_target_image<<<ctx->num_sms * 4, 256, 0, st>>>(F, c->L[0], c->L[1], c->L[2], b, box->lo[0], box->lo[1],
@@ -1048,7 +1127,12 @@ extern "C" mpm_status mpm_cnn_export_features(mpm_ctx *ctx, const mpm_cnn *c, in
         return mpm_fail(ctx, MPM_ERR_ARG, "cnn_export_features: bad argument");
     cudaStream_t st = (cudaStream_t)stream;
     const size_t n = (size_t)c->V * nimg;
-    MPM_CU(cudaMemcpyAsync(x_bf16, c->x, n * kXC * 2, cudaMemcpyDeviceToDevice, st));
+    if (((uintptr_t)x_bf16 & 15) == 0)
+        k_export_features<uint4><<<ctx->num_sms * 8, 256, 0, st>>>(c->x, c->mask, (int64_t)n, (uint4 *)x_bf16);
+    else
+        k_export_features<uint8_t><<<ctx->num_sms * 8, 256, 0, st>>>(c->x, c->mask, (int64_t)n, (uint8_t *)x_bf16);
+    ctx->launches += 1;
+    MPM_CU(cudaGetLastError());
     MPM_CU(cudaMemcpyAsync(mask, c->mask, n, cudaMemcpyDeviceToDevice, st));
     return MPM_OK;
 }
