@@ -22,6 +22,7 @@
 // the tensor cores read them from shared memory.
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstdio>
@@ -49,7 +50,7 @@ __host__ __device__ constexpr int dg_ci(int l) { return l == kLayers - 1 ? kGC6 
 
 __host__ __device__ constexpr int wimg_bytes(int ci, int no)
 {
-    return 9 * (3 * (ci / 8) + ((3 * (ci / 8)) & 1)) * (no / 8) * 128;
+    return 9 * (3 * (ci / 8) + ((3 * (ci / 8)) & 1)) * (no / 8) * 128;   // tc::WImg
 }
 
 // ---------------------------------------------------------------- weights
@@ -62,18 +63,19 @@ struct PrepArgs {
 };
 
 // Entry e (a bf16 element) of a weight image with input channels CI and N =
-// NO: core matrix cm = e / 64 at ((dy+1) * QP + q) * 3 NG + (dz+1) * NG + ng,
-// row r, column j.  Forward: value W[t][ci][co]; input gradient:
-// W[26 - t][co][ci] (the tap mirrored, input and output channels exchanged).
+// NO: core matrix cm = e / 64 at ((dy+1) * QP + p) * 3 NG + (dz+1) * NG + ng for
+// place p of the forward kernel's K order (tc::Stage), row r, column j.
+// Forward: value W[t][ci][co]; input gradient: W[26 - t][co][ci] (the tap
+// mirrored, input and output channels exchanged).
 __device__ float wimg_value(const float *W, int Ci, int Co, int CI, int NO, int e, bool dgrad)
 {
-    const int KC = CI / 8, QC = 3 * KC, QP = QC + (QC & 1), NG = NO / 8;
+    const int KC = CI / 8, QP = 3 * KC + ((3 * KC) & 1), NG = NO / 8;
     const int cm = e >> 6, w = e & 63, r = w >> 3, j = w & 7;
-    const int nn = cm % (3 * NG), rest = cm / (3 * NG);
-    const int q = rest % QP, dyi = rest / QP;
+    const int nn = cm % (3 * NG), p = cm / (3 * NG) % QP, dyi = cm / (3 * NG) / QP;
     const int dzi = nn / NG, ng = nn % NG;
-    if (q >= QC) return 0.0f;
-    const int c = q / KC, kc = q % KC;
+    const int col = CI == 24 ? tc::Stage<24>::column(p) : CI == 16 ? tc::Stage<16>::column(p) : tc::Stage<8>::column(p);
+    if (col < 0) return 0.0f;
+    const int c = col / KC, kc = col % KC;
     const int dx = c - 1, dy = dyi - 1, dz = dzi - 1;
     const int t = (dx + 1) + 3 * (dy + 1) + 9 * (dz + 1);
     const int n = ng * 8 + r, k = kc * 8 + j;   // output, input channel of this convolution
@@ -164,15 +166,15 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
 __device__ __forceinline__ bool unit_of(const CnnDom &D, uint32_t ci, Unit &u)
 {
     const uint32_t nsx = (D.L[0] + tc::kSlabX - 1) / tc::kSlabX, nsy = (D.L[1] + tc::kSlabY - 1) / tc::kSlabY;
-    const uint32_t nzs = (D.L[2] + tc::kZSeg - 1) / tc::kZSeg;
+    const uint32_t nzs = (D.L[2] + D.seg - 1) / D.seg;
     const uint32_t r1 = ci / nsx, r2 = r1 / nsy;
     const int i = (int)(ci - r1 * nsx), j = (int)(r1 - r2 * nsy), b = (int)(r2 / nzs);
     const int kz = (int)(r2 - (uint32_t)b * nzs);
     u.b = b;
     u.ox = D.lo[b][0] + i * tc::kSlabX;
     u.oy = D.lo[b][1] + j * tc::kSlabY;
-    u.z0 = D.lo[b][2] + kz * tc::kZSeg;
-    u.nz = min(tc::kZSeg, D.n[b][2] - kz * tc::kZSeg);
+    u.z0 = D.lo[b][2] + kz * D.seg;
+    u.nz = min(D.seg, D.n[b][2] - kz * D.seg);
     u.pad0 = u.pad1 = u.pad2 = 0;
     return i * tc::kSlabX < D.n[b][0] && j * tc::kSlabY < D.n[b][1] && u.nz > 0;
 }
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(1024) k_plan_compact(const __grid_constant__ C
 
 // Solver mode: the box of a subgrid (from device memory) on a lattice of dims
 // L.  Units are placed along y where the pleural space is: one warp per band
-// of the box (8 x columns by a segment of up to 8 depths) marks the band's
+// of the box (8 x columns by a segment of plan_seg depths) marks the band's
 // active tile rows (a row of the subgrid's tiles is active when a tile of it
 // overlapping the band is stored, i.e. holds an in-mask voxel) and starts a
 // unit of 16 rows at the first active tile row, the next one at the first
@@ -275,9 +277,11 @@ __global__ void __launch_bounds__(1024) k_plan_compact(const __grid_constant__ C
 __global__ void __launch_bounds__(256) k_plan_box(const BoxGeo *__restrict__ geo, const int32_t *__restrict__ tile_index,
                                                   int32_t L0, int32_t L1, int32_t L2, Unit *__restrict__ units,
                                                   int32_t *__restrict__ counters, int64_t max_units,
-                                                  CnnDom *__restrict__ dom_out, int32_t *__restrict__ err)
+                                                  CnnDom *__restrict__ dom_out, int32_t *__restrict__ err, int num_sms)
 {
     const BoxGeo g = *geo;
+    const int nxb = (g.n[0] + tc::kSlabX - 1) / tc::kSlabX, nyb = (g.n[1] + tc::kSlabY - 1) / tc::kSlabY;
+    const int seg = tc::plan_seg([&](int sg) { return (int64_t)nxb * nyb * ((g.n[2] + sg - 1) / sg); }, num_sms);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         CnnDom D;
         memset(&D, 0, sizeof(D));
@@ -285,6 +289,7 @@ __global__ void __launch_bounds__(256) k_plan_box(const BoxGeo *__restrict__ geo
         D.L[1] = L1;
         D.L[2] = L2;
         D.B = 1;
+        D.seg = seg;
         for (int d = 0; d < 3; ++d) {
             D.lo[0][d] = g.lo[d];
             D.n[0][d] = g.n[d];
@@ -292,15 +297,15 @@ __global__ void __launch_bounds__(256) k_plan_box(const BoxGeo *__restrict__ geo
         *dom_out = D;
     }
     if (g.n[0] <= 0) return;
-    const int nxb = (g.n[0] + tc::kSlabX - 1) / tc::kSlabX, nzs = (g.n[2] + tc::kZSeg - 1) / tc::kZSeg;
+    const int nzs = (g.n[2] + seg - 1) / seg;
     const int64_t nbands = (int64_t)nxb * nzs;
     const int lane = threadIdx.x & 31;
     const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nw = (gridDim.x * (int64_t)blockDim.x) >> 5;
     const int ty_n = g.nt[1], ly = g.lt[1];
     for (int64_t band = w0; band < nbands; band += nw) {
-        const int bx0 = (int)(band % nxb) * tc::kSlabX, bz0 = (int)(band / nxb) * tc::kZSeg;
-        const int nx = min(tc::kSlabX, g.n[0] - bx0), nz = min(tc::kZSeg, g.n[2] - bz0);
+        const int bx0 = (int)(band % nxb) * tc::kSlabX, bz0 = (int)(band / nxb) * seg;
+        const int nx = min(tc::kSlabX, g.n[0] - bx0), nz = min(seg, g.n[2] - bz0);
         const int tx0 = bx0 >> g.lt[0], tx1 = (bx0 + nx - 1) >> g.lt[0];
         const int tz0 = bz0 >> g.lt[2], tz1 = (bz0 + nz - 1) >> g.lt[2];
         int next_free = 0;                        // first box row no unit of this band covers
@@ -852,7 +857,13 @@ mpm_status plan_images(mpm_ctx *ctx, mpm_cnn *c, int nimg, cudaStream_t st)
 {
     CnnDom D = c->hdom;
     D.B = nimg;
-    const long long ncand = (long long)nimg * ((c->L[0] + 7) / 8) * ((c->L[1] + 15) / 16) * ((c->L[2] + 7) / 8);
+    D.seg = tc::plan_seg([&](int sg) {
+        int64_t n = 0;
+        for (int b = 0; b < nimg; ++b)
+            n += (int64_t)((D.n[b][0] + 7) / 8) * ((D.n[b][1] + 15) / 16) * ((D.n[b][2] + sg - 1) / sg);
+        return n;
+    }, ctx->num_sms);
+    const long long ncand = (long long)nimg * ((c->L[0] + 7) / 8) * ((c->L[1] + 15) / 16) * ((c->L[2] + D.seg - 1) / D.seg);
     MPM_CU(cudaMemsetAsync(c->counters, 0, 16 * sizeof(int32_t), st));
     k_plan_flags<<<ctx->num_sms * 4, 256, 0, st>>>(D, c->mask, ncand, c->flags);
     k_plan_compact<<<1, 1024, 0, st>>>(D, c->flags, ncand, c->units, c->counters, c->dom);
@@ -888,8 +899,12 @@ mpm_status forward_layers(mpm_ctx *ctx, mpm_cnn *c, const uint8_t *mask, bool tr
         if (l < kLayers - 1) {
             A.a_out = train ? c->a[l] : c->a[l & 1];
             A.z_out = train ? c->z[l] : nullptr;
-            r = l == 0 ? conv<kXC, 32, tc::EPI_GELU>(ctx, c, A, 1 + l, st)
-                       : conv<kHC, 32, tc::EPI_GELU>(ctx, c, A, 1 + l, st);
+            if (train)
+                r = l == 0 ? conv<kXC, 32, tc::EPI_TRAIN>(ctx, c, A, 1 + l, st)
+                           : conv<kHC, 32, tc::EPI_TRAIN>(ctx, c, A, 1 + l, st);
+            else
+                r = l == 0 ? conv<kXC, 32, tc::EPI_GELU>(ctx, c, A, 1 + l, st)
+                           : conv<kHC, 32, tc::EPI_GELU>(ctx, c, A, 1 + l, st);
         } else {
             tc::ConvArgs O = out_args;
             O.mask = mask;
@@ -962,9 +977,12 @@ extern "C" mpm_status mpm_cnn_create(mpm_ctx *ctx, mpm_cnn **out, const int32_t 
     c->nparams = n;
     const size_t VT = (size_t)V * max_images;
     // a band of 8 columns by 8 depths holds at most ceil(n_y / 16) units, on
-    // the fixed grid (image mode) and placed along y (solver mode) alike
-    c->max_units = (long long)max_images * ((image_dims[0] + 7) / 8) * ((image_dims[1] + 15) / 16) *
-                   ((image_dims[2] + 7) / 8);
+    // the fixed grid (image mode) and placed along y (solver mode) alike;
+    // shallower units (plan_seg) number fewer than twice the SMs.  The grid's
+    // candidates are counted over the whole image, at the shallowest depth.
+    const long long cols = (long long)max_images * ((image_dims[0] + 7) / 8) * ((image_dims[1] + 15) / 16);
+    c->max_units = std::max<long long>(cols * ((image_dims[2] + 7) / 8), 2LL * ctx->num_sms);
+    const long long max_cand = cols * ((image_dims[2] + 1) / 2);
     mpm_status r = MPM_OK;
     auto A = [&](void **p, size_t b) {
         if (r == MPM_OK) r = cnn_alloc(ctx, c, p, b);
@@ -995,7 +1013,7 @@ extern "C" mpm_status mpm_cnn_create(mpm_ctx *ctx, mpm_cnn **out, const int32_t 
     A((void **)&c->units, (size_t)c->max_units * sizeof(Unit));
     A((void **)&c->uact, (size_t)c->max_units * tc::kActStride);
     A((void **)&c->ubits, (size_t)c->max_units * sizeof(uint32_t));
-    A((void **)&c->flags, ((size_t)c->max_units + 15) & ~(size_t)15);   // read 16 bytes at a time
+    A((void **)&c->flags, ((size_t)max_cand + 15) & ~(size_t)15);   // read 16 bytes at a time
     A((void **)&c->counters, 64 * sizeof(int32_t));
     A((void **)&c->geo, 256);
     A((void **)&c->nact, 256);
@@ -1249,7 +1267,7 @@ mpm_status mpm_cnn_enqueue_guess(mpm_ctx *ctx, mpm_cnn *c, mpm_subgrid *sub, con
 {
     MPM_CU(cudaMemsetAsync(c->counters, 0, 16 * sizeof(int32_t), st));
     k_plan_box<<<ctx->num_sms, 256, 0, st>>>(d_geo, sub->tile_index, lat->dims[0], lat->dims[1], lat->dims[2], c->units,
-                                             c->counters, c->max_units, c->dom, c->d_err);
+                                             c->counters, c->max_units, c->dom, c->d_err, ctx->num_sms);
     ctx->launches += 1;
     mpm_status ra = unit_act(ctx, c, lat->mask, st);
     if (ra != MPM_OK) return ra;
@@ -1330,7 +1348,7 @@ mpm_status mpm_cnn_pc_plan(mpm_ctx *ctx, mpm_cnn *c, mpm_subgrid *sub, const mpm
     MPM_CU(cudaMemcpyAsync(c->geo, &g, sizeof(g), cudaMemcpyHostToDevice, st));
     MPM_CU(cudaMemsetAsync(c->counters, 0, 16 * sizeof(int32_t), st));
     k_plan_box<<<ctx->num_sms, 256, 0, st>>>(c->geo, sub->tile_index, lat->dims[0], lat->dims[1], lat->dims[2], c->units,
-                                             c->counters, c->max_units, c->dom, c->d_err);
+                                             c->counters, c->max_units, c->dom, c->d_err, ctx->num_sms);
     ctx->launches += 1;
     r = unit_act(ctx, c, lat->mask, st);
     if (r != MPM_OK) return r;

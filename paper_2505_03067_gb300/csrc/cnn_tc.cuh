@@ -10,21 +10,17 @@
 // and writes lattice-indexed buffers directly.
 //
 // Work decomposition.  The box of an image is cut into SLABS of 8 (x) x 16 (y)
-// x 1 (z) voxels -- M = 128 rows of one MMA -- and slabs into UNITS of kZSeg
+// x 1 (z) voxels -- M = 128 rows of one MMA -- and slabs into UNITS of up to kZSeg
 // consecutive slabs along z.  A plan kernel lists the units that hold an
 // active voxel; a persistent CTA per SM takes units from that list.
 //
 // Implicit GEMM.  For an output slab at depth z the convolution is
 //     D[v][co] = sum over (dy, dz) of sum over (dx, ci) of in[v + (dx,dy,dz)][ci] W[(dx,dy,dz)][ci][co].
-// The input halo of a depth (10 x 18 voxels) is staged in shared memory in
-// the tensor cores' canonical no-swizzle K-major layout with THREE copies
-// shifted by dx = -1, 0, +1 laid side by side along K: the core matrix of
-// K-column q = 3-copy index c times the channel chunks, plus the chunk kc,
-// for the 8 x-rows of halo row y', sits at y' * GS + q * 128.  A shift in y is
-// then a whole number of 8-row core-matrix groups, so the A operand of every
-// tap (dy, dz) is the same buffer at another start address: 9 taps x (K/16)
-// MMAs per slab read the staged halo in place, with no per-tap copy.  The
-// weights of all taps are staged once per CTA in the matching B layout.
+// The input halo of a depth (10 x 18 voxels) is staged in shared memory once, in
+// the tensor cores' no-swizzle K-major layout with the voxels of a row 16 bytes
+// apart (Stage): the A operand of every tap (dx, dy) is the same buffer at
+// another start address, with no per-tap copy.  The weights of all taps are
+// staged once per CTA in the matching B layout.
 //
 // Pipeline per CTA (forward kernel).  Loader warps copy halo depths with
 // cp.async (16 B, zero-filled for inactive voxels) into a ring of depth
@@ -58,7 +54,7 @@ constexpr int kHaloX = kSlabX + 2, kHaloY = kSlabY + 2;
 // nothing more, five less).
 constexpr int kEpiWarps = 12, kLoadWarps = 6;
 constexpr int kConvThreads = 32 * (kEpiWarps + kLoadWarps + 1);
-constexpr int kFwdSlots = 7;            // halo depths in the forward kernel's ring
+constexpr int kFwdSlots = 10;           // halo depths in the forward kernel's ring
 // TMEM of the forward kernel: two unit buffers of 256 columns, slab k of a
 // unit (k < kZSeg) accumulating in columns NO * (kZSeg - 1 - k) .. + NO of its
 // buffer (descending, so the slabs one input depth feeds are adjacent)
@@ -75,9 +71,25 @@ constexpr int kActStride = (kActBytes + 15) & ~15;
 struct CnnDom {
     int32_t L[3];                       // dims of one image
     int32_t B;                          // images
+    int32_t seg;                        // depths of a unit (2, 4 or kZSeg: plan_seg)
     int32_t lo[kMaxImages][3];          // box of each image
     int32_t n[kMaxImages][3];           // (n[b][0] == 0: empty image)
 };
+
+// Depths of a unit.  A unit's halves in z share nothing but two halo depths, so
+// deep units load least; but a box of fewer units than SMs leaves SMs idle and
+// each layer as long as one deep unit.  So the depth is halved while all boxes
+// together have fewer units than SMs: a 32^3 box has 32 units of 8 depths (ten
+// input depths one after the other) or 128 of 2 (four): flexible GMRES on it,
+// a chain of such layers, takes 1373 us a solve against 1729.
+// units(seg): an upper bound of the units of depth seg.
+template <typename F>
+__host__ __device__ __forceinline__ int plan_seg(F &&units, int num_sms)
+{
+    int seg = kZSeg;
+    while (seg > 2 && units(seg) < num_sms) seg >>= 1;
+    return seg;
+}
 
 // A unit: image b, slab origin (ox, oy) in image coordinates, depths
 // [z0, z0 + nz) (nz <= kZSeg).
@@ -177,18 +189,7 @@ __device__ __forceinline__ void tmem_zero8(uint32_t taddr)
     asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr), "r"(0u)
                  : "memory");
 }
-__device__ __forceinline__ void tmem_zero1(uint32_t taddr)
-{
-    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(0u) : "memory");
-}
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
-
-__device__ __forceinline__ float tmem_ld1(uint32_t taddr)
-{
-    uint32_t r;
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(r) : "r"(taddr));
-    return __uint_as_float(r);
-}
 
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8])
 {
@@ -207,6 +208,11 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint32
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
+// The same past L1, for chunks read once.
+__device__ __forceinline__ void cp_async16_cg(uint32_t dst, const void *src, uint32_t src_bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
 // Wait for every copy this thread issued.
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
@@ -216,7 +222,28 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 // erf(x) = 1 - (a1 t + a2 t^2 + a3 t^3 + a4 t^4 + a5 t^5) exp(-x^2), t = 1 / (1 + p x).
 // For z < 0, Phi(z) = (1 - erf(|z| / sqrt 2)) / 2.  Far below the bf16 rounding
 // of the stored activation (2^-9 relative).
+// The reciprocal is the hardware's approximation with one Newton step, 2^-y^2 the
+// hardware's exponential: 18 instructions an element (27 with __frcp_rn and
+// exp2f, which guard ranges that do not occur here); the epilogue's
+// instructions compete with the loaders' and the MMA warp's for issue slots.
+// The clamp keeps the Newton step finite: GELU(+inf) = inf, GELU(-inf) = NaN.
 __device__ __forceinline__ float gelu(float z)
+{
+    const float a = fminf(fabsf(z), 1e4f);
+    const float d = fmaf(0.3275911f * 0.70710678118654752f, a, 1.0f);
+    float t, e;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(t) : "f"(d));
+    t = fmaf(t, fmaf(-d, t, 1.0f), t);
+    const float y = a * 0.84932180028801905f;             // y^2 = z^2 / 2 * log2 e
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-(y * y)));
+    const float poly = t * fmaf(t, fmaf(t, fmaf(t, fmaf(t, 0.5f * 1.061405429f, 0.5f * -1.453152027f), 0.5f * 1.421413741f),
+                                        0.5f * -0.284496736f), 0.5f * 0.254829592f);
+    const float half_tail = poly * e;                     // (1 - erf(x)) / 2
+    return z * (z >= 0.0f ? 1.0f - half_tail : half_tail);
+}
+// The same with the reciprocal rounded to nearest and the library's exponential:
+// the training steps' form, whose last bits Adam's first steps would amplify.
+__device__ __forceinline__ float gelu_train(float z)
 {
     const float x = fabsf(z) * 0.70710678118654752f;
     const float t = __frcp_rn(fmaf(0.3275911f, x, 1.0f));
@@ -244,15 +271,52 @@ struct Halo {
     static constexpr int NKS = QP / 2;             // MMAs of K = 16 per tap
 };
 
-// Weight image of one layer for the forward kernel: for tap row dy, K-column
-// q, tap depth dz and output-channel group ng, the 8 x 8 core matrix (rows n =
-// ng*8 + r, columns k = q*8 + j) at (((dy+1) * QP + q) * 3 NG + (dz+1) * NG +
-// ng) * 128 bytes: the three depths' N blocks are adjacent, so one MMA of N =
-// 3 NO applies the taps dz = -1, 0, +1 of an input depth to three output slabs.
+// The forward kernel's staged halo depth: the voxels once, [halo row y'][chunk
+// kc][halo column x'][8 channels].  A core matrix of a no-swizzle K-major operand
+// is eight rows of 16 contiguous bytes at any 16-byte address, so the matrix of
+// tap column dx starts 16 (dx + 1) bytes into its chunk's row of ten voxels: the
+// three shifts along x read one copy at overlapping addresses, as the shifts
+// along y read it at other rows.  The K-columns of one MMA (K = 16) are two core
+// matrices at a constant positive distance (LBO): per tap row the columns go by
+// (dx, kc), the pair that would run backwards is exchanged, and an odd last one
+// is paired with the matrix before it under zero weights (its values are in the
+// tap window, so a value that is not finite spoils nothing it would not anyway).
+// Each MMA sums the same products as with three shifted copies side by side
+// (which the weight gradient still needs), so the sums are the same bit for
+// bit; a depth takes 540 copies of 16 bytes instead of 1296.  Fewer MMAs a depth
+// (14 of 15, pairs across tap rows) gave 2 % and changed the sums' order, and
+// with it training: Adam's first steps turn a last-bit change of a gradient
+// near zero into a whole step.
+template <int CI>
+struct Stage {
+    static constexpr int KC = CI / 8;
+    static constexpr int QC = 3 * KC;              // columns of a tap row: q = (dx + 1) * KC + kc
+    static constexpr int QP = QC + (QC & 1);       // places of a tap row's K order
+    static constexpr int NMMA = 3 * QP / 2;        // MMAs of a depth
+    static constexpr int XS = kHaloX * 16;         // bytes of a chunk's row
+    static constexpr int YS = KC * XS;             // bytes of a halo row
+    static constexpr int SLOT = kHaloY * YS;       // bytes of a depth
+    __host__ __device__ static constexpr int column_offset(int q) { return q % KC * XS + q / KC * 16; }
+    // column in place p of the K order; -1: zero weights
+    __host__ __device__ static constexpr int column(int p)
+    {
+        return QP > QC && p >= QC - 1 ? (p == QC - 1 ? -1 : QC - 1)
+                                      : (column_offset(p | 1) < column_offset(p & ~1) ? p ^ 1 : p);
+    }
+    // byte offset in its halo row of the core matrix in place p (zero weights: the matrix before the last)
+    __host__ __device__ static constexpr int offset(int p) { return column_offset(column(p) < 0 ? QC - 2 : column(p)); }
+};
+
+// Weight image of one layer for the forward kernel: for tap row dy, place p of
+// the K order (Stage), tap depth dz and output-channel group ng, the 8 x 8 core
+// matrix (rows n = ng*8 + r, columns the place's 8 channels) at (((dy+1) * QP +
+// p) * 3 NG + (dz+1) * NG + ng) * 128 bytes: the three depths' N blocks are
+// adjacent, so one MMA of N = 3 NO applies the taps dz = -1, 0, +1 of an input
+// depth to three output slabs.
 template <int CI, int NO>
 struct WImg {
     static constexpr int NG = NO / 8;
-    static constexpr int BYTES = 9 * Halo<CI>::QP * NG * 128;
+    static constexpr int BYTES = 9 * Stage<CI>::QP * NG * 128;
 };
 
 // Shared memory of the forward kernel.
@@ -260,7 +324,7 @@ template <int CI, int NO>
 struct ConvSmem {
     static constexpr int W_OFF = 0;
     static constexpr int RING_OFF = (WImg<CI, NO>::BYTES + 1023) & ~1023;
-    static constexpr int RING_BYTES = kFwdSlots * Halo<CI>::SLOT;
+    static constexpr int RING_BYTES = (kFwdSlots * Stage<CI>::SLOT + 15) & ~15;
     static constexpr int ACT_BYTES = kActStride;
     static constexpr int ACT_OFF = RING_OFF + RING_BYTES;          // two units' activity bytes
     static constexpr int UNIT_OFF = (ACT_OFF + 2 * ACT_BYTES + 15) & ~15;   // two Units + two slab masks
@@ -273,7 +337,7 @@ struct ConvSmem {
     static constexpr int BYTES = BYTES0 > 120 * 1024 ? BYTES0 : 120 * 1024;
 };
 
-enum { EPI_GELU = 0, EPI_OUT = 1, EPI_DGRAD = 2 };
+enum { EPI_GELU = 0, EPI_OUT = 1, EPI_DGRAD = 2, EPI_TRAIN = 3 };
 
 struct ConvArgs {
     const __nv_bfloat16 *in;        // [B * V][CI]
@@ -287,7 +351,7 @@ struct ConvArgs {
     int32_t *done;                  //   CTAs finished (reset with it)
     const unsigned char *wimg;      // weight image (WImg layout)
     const float *bias;              // [NO] (null: none)
-    // EPI_GELU: a_out = bf16(gelu(z)) at active voxels, z_out (nullable) = z
+    // EPI_GELU, EPI_TRAIN: a_out = bf16(gelu(z)) at active voxels; EPI_TRAIN: z_out = z
     __nv_bfloat16 *a_out;           // [B * V][24]
     float *z_out;                   // [B * V][24]
     // EPI_OUT: pred = c^n + s_out * z (3 channels)
@@ -407,6 +471,48 @@ __device__ __forceinline__ uint32_t row_bits(const uint8_t *__restrict__ mask, i
     return bits & ((1u << (xe - x0)) - 1u) & ~((1u << (xs - x0)) - 1u);
 }
 
+// The forward kernel's copies of one halo depth, likewise: item i is chunk kc of
+// halo voxel (x', y'), kc fastest, so a warp reads 512 contiguous bytes of the
+// source rows (a voxel's chunks are adjacent there).
+template <int CI, int NL>
+struct StageItems {
+    using H = Stage<CI>;
+    static constexpr int N = kHaloY * kHaloX * H::KC;
+    static constexpr int K = (N + NL - 1) / NL;
+    int32_t rel[K];
+    uint32_t da[K];                 // shared offset (low 16 bits), activity index (255: no item)
+    __device__ __forceinline__ void init(int tid, int L0)
+    {
+        static_assert(kHaloY * kHaloX < 255 && H::SLOT < 65536, "packed halo item");
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+            const int i = tid + k * NL;
+            const int kc = i % H::KC, v = i / H::KC;
+            const int xh = v % kHaloX, yh = v / kHaloX;
+            rel[k] = (yh * L0 + xh) * CI + kc * 8;
+            da[k] = (uint32_t)(yh * H::YS + kc * H::XS + xh * 16) | ((i < N ? (uint32_t)v : 255u) << 16);
+        }
+    }
+};
+
+// cp.async the halo depth j of unit u into slot base `dst` (zero-filled where
+// inactive); every chunk is read once, so the copies bypass L1.
+template <int CI, int NL>
+__device__ __forceinline__ void load_stage_depth(const CnnDom &D, const __nv_bfloat16 *__restrict__ in, const Unit &u,
+                                                 const uint8_t *act, int j, uint32_t dst, const StageItems<CI, NL> &it)
+{
+    const uint8_t *aj = act + j * kHaloY * kHaloX;
+    const int64_t base = (((int64_t)u.b * D.L[2] + (u.z0 - 1 + j)) * D.L[1] + (u.oy - 1)) * (int64_t)D.L[0] + (u.ox - 1);
+#pragma unroll
+    for (int k = 0; k < StageItems<CI, NL>::K; ++k) {
+        const uint32_t ai = it.da[k] >> 16;
+        if (ai == 255u) continue;
+        const bool ok = aj[ai] != 0;
+        const __nv_bfloat16 *src = ok ? in + (base * CI + it.rel[k]) : in;
+        cp_async16_cg(dst + (it.da[k] & 0xFFFFu), src, ok ? 16u : 0u);
+    }
+}
+
 // One CTA per listed unit (grid-strided): its activity bytes and slab mask, a
 // thread per row of ten voxels (three or four words in flight).  Bound by the
 // latency of unit record and mask, so eight CTAs an SM; one thread per byte
@@ -518,21 +624,20 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t *bar, uint32_t parity, u
 //    slots (cp.async; a slot's mbarrier completes when every loader's copies
 //    into it have landed; a slot is refilled once the MMAs that read it
 //    completed);
-//  - 1 MMA warp (one elected lane) issues, per input depth, 3 tap rows (dy) x
-//    (K/16) MMAs of N = up to 3 NO: the depth's halo (the A operand, read
+//  - 1 MMA warp (one elected lane) issues, per input depth, the tap rows' and
+//    columns' MMAs of N = up to 3 NO: the depth's halo (the A operand, read
 //    once) times the weights of its three tap depths dz, accumulating into
 //    the accumulators of the (active) output slabs it feeds, which lie side
 //    by side in TMEM and start at zero.  A commit releases the depth's ring
 //    slot, and one marks slab j - 2 complete after depth j;
-//  - 12 EPILOGUE warps (warp w: TMEM lane quarter w & 3, channels
-//    8 (w >> 2) .. 8 (w >> 2) + 7; the output layer: channel w >> 2) drain
-//    each complete slab through the epilogue, zero their columns of the
-//    unit's TMEM buffer and hand it back.
+//  - 12 EPILOGUE warps (warp w: TMEM lane quarter w & 3; the group w >> 2
+//    takes every third slab, or 8 channels of every slab) drain the complete
+//    slabs, zero their columns of the unit's TMEM buffer and hand it back.
 // NO: MMA N (output channels padded to 16 or 32).
 template <int CI, int NO, int EPI>
 __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
 {
-    using H = Halo<CI>;
+    using H = Stage<CI>;
     using S = ConvSmem<CI, NO>;
     constexpr int NG = WImg<CI, NO>::NG;
     constexpr int NE = 32 * kEpiWarps;            // epilogue threads: 0 .. NE-1
@@ -550,11 +655,9 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
     const uint32_t wbase = smem_u32(sm + S::W_OFF), rbase = smem_u32(sm + S::RING_OFF);
     volatile int32_t *abort = &s_abort;
 
-    // weights into shared memory; zero the ring (pad K-columns stay zero)
+    // weights into shared memory
     for (int i = tid; i < WImg<CI, NO>::BYTES / 16; i += kConvThreads)
         reinterpret_cast<uint4 *>(sm + S::W_OFF)[i] = __ldg(reinterpret_cast<const uint4 *>(A.wimg) + i);
-    for (int i = tid; i < S::RING_BYTES / 16; i += kConvThreads)
-        reinterpret_cast<uint4 *>(sm + S::RING_OFF)[i] = make_uint4(0u, 0u, 0u, 0u);
     if (warp == 0) tmem_alloc(&s_tmem, 2 * kTmemBuf);
     if (tid == 0) {
         s_abort = 0;
@@ -600,14 +703,16 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
         // outcome (s_lstop) before a named barrier, so every decision of the
         // loader warps is uniform.
         const int lt = tid - NE;
-        HaloItems<CI, NLD> items;
+        StageItems<CI, NLD> items;
         items.init(lt, D.L[0]);
         // Units are taken from a counter shared by the CTAs (units hold 1..8
         // active slabs, so a fixed assignment leaves CTAs unequally loaded).
-        // The next unit's index, activity bytes (one 16-byte share per
-        // thread), record and slab mask are fetched a unit ahead, so a unit's
-        // start waits on no global round trip; an index past the list is
-        // published as the stop record.
+        // The next unit's index is drawn two units ahead, its activity bytes
+        // (one 16-byte share per thread), record and slab mask are fetched a
+        // unit ahead, so a unit's start waits on no global round trip (drawn
+        // one unit ahead, the atomic's round trip stood between the units:
+        // ~5000 of ~14 500 cycles a unit); an index past the list is published
+        // as the stop record.
         constexpr int kAct16 = kActStride / 16;
         static_assert(kAct16 <= NLD, "one activity share per loader thread");
         const uint4 *uact4 = reinterpret_cast<const uint4 *>(A.uact);
@@ -615,7 +720,11 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
         Unit urow;
         urow.b = urow.ox = urow.oy = urow.z0 = urow.nz = urow.pad0 = urow.pad1 = urow.pad2 = 0;
         uint32_t ubit = 0u;
-        if (lt == 0) s_ui = atomicAdd(A.work, 1);
+        int drawn = 0;                            // loader 0: the unit after the next
+        if (lt == 0) {
+            s_ui = atomicAdd(A.work, 1);
+            drawn = atomicAdd(A.work, 1);
+        }
         named_sync(1, NLD);
         int ui = s_ui;
         if (ui < nunits) {
@@ -630,7 +739,8 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
             const int ub = n & 1;
             named_sync(1, NLD);                   // every loader read s_ui
             if (lt == 0) {
-                s_ui = ui < nunits ? atomicAdd(A.work, 1) : nunits;
+                s_ui = ui < nunits ? drawn : nunits;
+                if (ui < nunits && drawn < nunits) drawn = atomicAdd(A.work, 1);   // read at the next unit
                 const bool w = n < 2 || mbar_wait_or_abort(&unite[ub], ((n >> 1) - 1) & 1, T, A.err, abort);
                 if (!w || *abort) s_lstop = 1;
             }
@@ -669,7 +779,7 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
                     s_lstop = 1;
                 named_sync(1, NLD);
                 if (s_lstop) break;
-                load_halo_depth_items<CI, NLD>(D, A.in, u, act, j, rbase + slot * H::SLOT, items);
+                load_stage_depth<CI, NLD>(D, A.in, u, act, j, rbase + slot * H::SLOT, items);
                 cp_async_arrive(&full[slot]);   // completes the slot's phase once the copies land
                 ++dseq;
             }
@@ -685,8 +795,8 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
         constexpr uint32_t kId1 = idesc_bf16(128, NO, false, false), kId2 = idesc_bf16(128, 2 * NO, false, false),
                            kId3 = idesc_bf16(128, 3 * NO, false, false);
         const uint32_t tm = __shfl_sync(0xffffffffu, tmem, 0);
-        const uint32_t alo0 = sdesc_lo(rbase, 128u), blo0 = sdesc_lo(wbase, 3u * NG * 128u);
-        constexpr uint32_t ahi = sdesc_hi(H::GS), bhi = sdesc_hi(128u);
+        const uint32_t alo0 = sdesc_lo(rbase, 0u), blo0 = sdesc_lo(wbase, 3u * NG * 128u);
+        constexpr uint32_t ahi = sdesc_hi(H::YS), bhi = sdesc_hi(128u);
         uint32_t dbase = 0;
         bool ok = true;
         for (int n = 0; ok; ++n) {
@@ -721,11 +831,14 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
                     const uint32_t blo = blo0 + (uint32_t)((j - hi) * NG * 8);
                     // the accumulators start at zero (see the epilogue), so every MMA accumulates
 #pragma unroll
-                    for (int t = 0; t < 3 * H::NKS; ++t) {
-                        const int dyi = t / H::NKS, s2 = t % H::NKS;
-                        // A: halo row dyi, K-columns 2 s2 .. 2 s2 + 1; B: core matrix (dy, q = 2 s2, dz block j - hi, ng 0)
-                        mma_bf16_warp(dacc, alo + (uint32_t)((dyi * H::GS) >> 4) + (uint32_t)(s2 * 16), ahi,
-                                      blo + (uint32_t)((dyi * H::QP + 2 * s2) * 3 * NG * 8), bhi, idn, 1u);
+                    for (int t = 0; t < H::NMMA; ++t) {
+                        // A: halo row dyi, places p and p + 1 of the K order, LBO their distance;
+                        // B: their core matrices of dz block j - hi, ng 0
+                        const int dyi = 2 * t / H::QP, p = 2 * t % H::QP;
+                        const uint32_t off = (uint32_t)(dyi * H::YS + H::offset(p)) >> 4;
+                        const uint32_t lbo = (uint32_t)(H::offset(p + 1) - H::offset(p)) >> 4;
+                        mma_bf16_warp(dacc, alo + off + (lbo << 16), ahi, blo + (uint32_t)(2 * t * 3 * NG * 8), bhi, idn,
+                                      1u);
                     }
                 }
                 mma_commit_warp(&empty[slot]);          // no later MMA reads this depth
@@ -741,22 +854,29 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
         __syncwarp();
     } else if (tid < NE) {
         // ------------------------------------------------------------ epilogue
+        // Warp w reads the TMEM lane quarter w & 3.  A forward layer's slabs go
+        // round the three warp groups w >> 2, each draining all channels of its
+        // slabs (the fixed part of a slab -- waits, activity, addresses -- once
+        // per voxel, 24 independent GELUs in flight).  With 8 channels of every
+        // slab a group the epilogue held the kernel back (busy 75 % of the time
+        // beside MMAs busy 60 %): a hidden layer of a 324x264x264 shell took 252
+        // us and takes 217, bound by the MMAs' issue.  The input gradient's
+        // pre-activations would not fit the registers that way, so there every
+        // group takes 8 channels of every slab.
+        constexpr bool kBySlab = EPI != EPI_DGRAD;
+        constexpr int NCH = EPI == EPI_OUT ? 3 : (kBySlab ? 24 : 8);   // channels of a thread
+        constexpr int NCG = EPI == EPI_OUT ? 1 : NCH / 8;
         const int lq = warp & 3, wq = warp >> 2;
         const int row = lq * 32 + lane;           // voxel (row & 7, row >> 3) of the slab
         const int ex = row & 7, ey = row >> 3;
-        // first channel of this thread: 8 channels per warp group; the output
-        // layer's three channels go one to each warp group (channel wq)
-        const int c0 = EPI == EPI_OUT ? wq : 8 * wq;
+        const int c0 = kBySlab ? 0 : 8 * wq;      // first channel of this thread
+        const int kfirst = kBySlab ? wq : 0;
+        constexpr int kstep = kBySlab ? 3 : 1;
         // (image mode writes all three predicted channels, solver mode the species')
-        const bool reads = EPI != EPI_OUT || wq < (A.pred ? 3 : (A.nspecies < 3 ? A.nspecies : 3));
-        float bias[8];
+        const int nout = A.pred ? 3 : (A.nspecies < 3 ? A.nspecies : 3);
+        float bias[NCH];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) bias[i] = 0.0f;
-        if (A.bias && EPI != EPI_DGRAD) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i)
-                if (EPI != EPI_OUT || i == 0) bias[i] = A.bias[c0 + i];
-        }
+        for (int i = 0; i < NCH; ++i) bias[i] = A.bias && EPI != EPI_DGRAD ? A.bias[c0 + i] : 0.0f;
         bool ok = true;
         for (int n = 0; ok; ++n) {
             const int ub = n & 1;
@@ -767,26 +887,35 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
             if (u.nz < 0) break;                  // the stop record
             const uint32_t bits = ubits[ub];
             const uint8_t *act = sm + S::ACT_OFF + ub * S::ACT_BYTES;
-            for (int k = 0; k < u.nz && ok; ++k) {
-                if (!((bits >> k) & 1u)) continue;
+            const uint32_t tbuf = tmem + (uint32_t)ub * kTmemBuf + ((uint32_t)(lq * 32) << 16);
+            // a group without a slab in this unit still waits for one (the
+            // parities of its later waits rest on having passed every unit)
+            if (kfirst >= u.nz) ok = mbar_wait_warp(&accf[ub * kZSeg], (n >> 1) & 1, T, A.err, abort);
+            for (int k = kfirst; k < u.nz && ok; k += kstep) {
+                const bool live = (bits >> k) & 1u;
                 const int z = u.z0 + k, x = u.ox + ex, y = u.oy + ey;
-                const bool on = reads && act[((k + 1) * kHaloY + ey + 1) * kHaloX + ex + 1] != 0;
+                const bool on = live && act[((k + 1) * kHaloY + ey + 1) * kHaloX + ex + 1] != 0;
                 const int64_t v = on ? vox_index(D, u.b, x, y, z) : 0;
                 // operands that do not depend on the MMAs: loaded before the wait
-                float pre[8];
+                float pre[NCH];
                 int64_t e = -1;
                 double cn[3] = {0.0, 0.0, 0.0};
+                if (EPI == EPI_DGRAD || EPI == EPI_OUT) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) pre[i] = 0.0f;
+                    for (int i = 0; i < NCH; ++i) pre[i] = 0.0f;
+                }
                 if (on) {
                     if (EPI == EPI_DGRAD) {
                         const float4 *zp = reinterpret_cast<const float4 *>(A.zprev + v * 24 + c0);
-                        const float4 q0 = zp[0], q1 = zp[1];
-                        pre[0] = q0.x; pre[1] = q0.y; pre[2] = q0.z; pre[3] = q0.w;
-                        pre[4] = q1.x; pre[5] = q1.y; pre[6] = q1.z; pre[7] = q1.w;
+#pragma unroll
+                        for (int i = 0; i < NCG * 2; ++i) {
+                            const float4 q = zp[i];
+                            pre[4 * i] = q.x; pre[4 * i + 1] = q.y; pre[4 * i + 2] = q.z; pre[4 * i + 3] = q.w;
+                        }
                     } else if (EPI == EPI_OUT) {
                         if (A.pred) {
-                            pre[0] = A.f32[v * 3 + c0];
+#pragma unroll
+                            for (int c = 0; c < NCH; ++c) pre[c] = A.f32[v * 3 + c];
                         } else {
                             const BoxGeo &g = *A.geo;
                             const int bx = x - g.lo[0], by = y - g.lo[1], bz = z - g.lo[2];
@@ -797,7 +926,9 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
                                           iz = bz & ((1 << g.lt[2]) - 1);
                                 e = ((int64_t)t << (g.lt[0] + g.lt[1] + g.lt[2])) + ix +
                                     ((int64_t)(iy + (iz << g.lt[1])) << g.lt[0]);
-                                cn[0] = A.field[c0][v];
+#pragma unroll
+                                for (int c = 0; c < 3; ++c)
+                                    if (c < nout) cn[c] = A.field[c][v];
                             }
                         }
                     }
@@ -805,67 +936,66 @@ __global__ void __maxnreg__(96) k_conv_tc(const __grid_constant__ ConvArgs A)
                 ok = mbar_wait_warp(&accf[ub * kZSeg + k], (n >> 1) & 1, T, A.err, abort);
                 if (!ok) break;
                 tc_after_sync();
-                float d[8];
-                if (reads) {
-                    const uint32_t ta = tmem + (uint32_t)ub * kTmemBuf + (uint32_t)(NO * (kZSeg - 1 - k)) + (uint32_t)c0 +
-                                        ((uint32_t)(lq * 32) << 16);
-                    if (EPI == EPI_OUT)
-                        d[0] = tmem_ld1(ta);
-                    else
-                        tmem_ld8(ta, d);
+                const uint32_t ta = tbuf + (uint32_t)(NO * (kZSeg - 1 - k)) + (uint32_t)c0;
+                float d[NCG][8];
+                if (live) {
+#pragma unroll
+                    for (int g = 0; g < NCG; ++g) tmem_ld8(ta + 8 * g, d[g]);
                     tc_wait_ld();
                 }
+                // the columns start the buffer's next unit from zero (every MMA
+                // accumulates; an inactive slab between active ones was written too)
+#pragma unroll
+                for (int g = 0; g < NCG; ++g) tmem_zero8(ta + 8 * g);
                 if (on) {
                     if (EPI == EPI_OUT) {
                         if (A.pred) {
-                            A.pred[v * 3 + c0] = pre[0] + A.s_out * (d[0] + bias[0]);
+#pragma unroll
+                            for (int c = 0; c < NCH; ++c)
+                                A.pred[v * 3 + c] = pre[c] + A.s_out * (d[0][c] + bias[c]);
                         } else if (e >= 0) {
-                            const double p = cn[0] + (double)(A.s_out * (d[0] + bias[0]));
-                            A.xs[c0][e] = isfinite(p) ? p : cn[0];   // a non-finite guess falls back to c^n
+#pragma unroll
+                            for (int c = 0; c < NCH; ++c) {
+                                if (c >= nout) break;
+                                const double p = cn[c] + (double)(A.s_out * (d[0][c] + bias[c]));
+                                A.xs[c][e] = isfinite(p) ? p : cn[c];   // a non-finite guess falls back to c^n
+                            }
                         }
                     } else {
-                        uint32_t o[4];
-                        if (EPI == EPI_GELU) {
-                            float zz[8];
 #pragma unroll
-                            for (int c = 0; c < 8; ++c) zz[c] = d[c] + bias[c];
-                            if (A.z_out) {
-                                float4 *zp = reinterpret_cast<float4 *>(A.z_out + v * 24 + c0);
-                                zp[0] = make_float4(zz[0], zz[1], zz[2], zz[3]);
-                                zp[1] = make_float4(zz[4], zz[5], zz[6], zz[7]);
-                            }
+                        for (int g = 0; g < NCG; ++g) {
+                            uint32_t o[4];
+                            float(&dd)[8] = d[g];
+                            if (EPI == EPI_GELU || EPI == EPI_TRAIN) {
 #pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                __nv_bfloat162 h = __floats2bfloat162_rn(gelu(zz[2 * c]), gelu(zz[2 * c + 1]));
-                                o[c] = *reinterpret_cast<uint32_t *>(&h);
-                            }
-                            *reinterpret_cast<uint4 *>(A.a_out + v * 24 + c0) = make_uint4(o[0], o[1], o[2], o[3]);
-                        } else {   // EPI_DGRAD
+                                for (int c = 0; c < 8; ++c) dd[c] += bias[8 * g + c];
+                                if (EPI == EPI_TRAIN) {
+                                    float4 *zp = reinterpret_cast<float4 *>(A.z_out + v * 24 + c0 + 8 * g);
+                                    zp[0] = make_float4(dd[0], dd[1], dd[2], dd[3]);
+                                    zp[1] = make_float4(dd[4], dd[5], dd[6], dd[7]);
+                                }
 #pragma unroll
-                            for (int c = 0; c < 4; ++c) {
-                                __nv_bfloat162 h = __floats2bfloat162_rn(d[2 * c] * gelu_grad(pre[2 * c]),
-                                                                         d[2 * c + 1] * gelu_grad(pre[2 * c + 1]));
-                                o[c] = *reinterpret_cast<uint32_t *>(&h);
+                                for (int c = 0; c < 4; ++c) {
+                                    __nv_bfloat162 h = EPI == EPI_TRAIN ? __floats2bfloat162_rn(gelu_train(dd[2 * c]), gelu_train(dd[2 * c + 1]))
+                                                       : __floats2bfloat162_rn(gelu(dd[2 * c]), gelu(dd[2 * c + 1]));
+                                    o[c] = *reinterpret_cast<uint32_t *>(&h);
+                                }
+                                *reinterpret_cast<uint4 *>(A.a_out + v * 24 + c0 + 8 * g) = make_uint4(o[0], o[1], o[2], o[3]);
+                            } else {   // EPI_DGRAD
+                                const float *pr = pre + 8 * (EPI == EPI_DGRAD ? g : 0);
+#pragma unroll
+                                for (int c = 0; c < 4; ++c) {
+                                    __nv_bfloat162 h = __floats2bfloat162_rn(dd[2 * c] * gelu_grad(pr[2 * c]),
+                                                                             dd[2 * c + 1] * gelu_grad(pr[2 * c + 1]));
+                                    o[c] = *reinterpret_cast<uint32_t *>(&h);
+                                }
+                                *reinterpret_cast<uint4 *>(A.g_out + v * 24 + c0 + 8 * g) = make_uint4(o[0], o[1], o[2], o[3]);
                             }
-                            *reinterpret_cast<uint4 *>(A.g_out + v * 24 + c0) = make_uint4(o[0], o[1], o[2], o[3]);
                         }
                     }
                 }
             }
-            // zero this warp's accumulator columns of every slab of the buffer
-            // (every MMA accumulates; unit n + 2 starts from these zeros): all
-            // MMAs into the buffer completed with its last active slab
-            if (ok) {
-                const uint32_t tq = tmem + (uint32_t)ub * kTmemBuf + (uint32_t)c0 + ((uint32_t)(lq * 32) << 16);
-#pragma unroll
-                for (int k = 0; k < kZSeg; ++k) {
-                    if (EPI == EPI_OUT)
-                        tmem_zero1(tq + (uint32_t)(NO * (kZSeg - 1 - k)));
-                    else
-                        tmem_zero8(tq + (uint32_t)(NO * (kZSeg - 1 - k)));
-                }
-                tc_wait_st();
-            }
+            if (ok) tc_wait_st();
             // this warp is done with the unit's TMEM buffer, activity bytes and records
             tc_before_sync();
             __syncwarp();
