@@ -30,6 +30,9 @@ struct AsmArgs {
 // diffusivity factors come from the compact copy through the tile table.
 __global__ void __launch_bounds__(kBlock) k_assemble(AsmArgs A, int64_t NE)
 {
+    __shared__ RowCoef R;
+    if ((int)threadIdx.x < A.C.nspecies) R.init(A.C, threadIdx.x);
+    __syncthreads();
     const int ltv = A.lt[0] + A.lt[1] + A.lt[2];
     for (int64_t e = (int64_t)blockIdx.x * kBlock + threadIdx.x; e < NE; e += (int64_t)gridDim.x * kBlock) {
         const uint32_t f = A.flags[e];
@@ -80,7 +83,7 @@ __global__ void __launch_bounds__(kBlock) k_assemble(AsmArgs A, int64_t NE)
             for (int d = 0; d < 6; ++d) A.hm[d * A.hstride + e] = hm[d];
         for (int s = 0; s < A.C.nspecies; ++s) {
             double dg, b;
-            assemble_row(A.C, s, f, id, ndir, A.dfac != nullptr, fp, hsum, A.cn[s][e], dg, b);
+            assemble_row(A.C, &R, s, f, id, ndir, A.dfac != nullptr, fp, hsum, A.cn[s][e], dg, b);
             A.diag[s][e] = dg;
             A.diag32[s][e] = f32_rz(dg);
             A.b[s][e] = b;

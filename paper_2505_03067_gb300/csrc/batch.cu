@@ -56,10 +56,13 @@ __global__ void __launch_bounds__(kBlock) k_batch_prep(const char *__restrict__ 
     const BatchSys &S = reinterpret_cast<const BatchSys *>(buf + desc_off(nsys))[i];
     const int64_t e0 = (blockIdx.x - blk0[i]) * (int64_t)(kBlock * kEPT);
     const int64_t e1 = min(S.NE, e0 + (int64_t)(kBlock * kEPT));
+    __shared__ RowCoef R;
+    if ((int)threadIdx.x < S.C.nspecies) R.init(S.C, threadIdx.x);
+    __syncthreads();
     const BoxGeo g = S.g;
     for (int64_t e = e0 + threadIdx.x; e < e1; e += kBlock) {
-        if (kVar) prep_elem<false>(S, g, e);
-        else prep_elem_t<false, false>(S, g, e, nullptr, nullptr, nullptr);
+        if (kVar) prep_elem<false>(S, g, e, &R);
+        else prep_elem_t<false, false>(S, g, e, &R, nullptr, nullptr, nullptr);
     }
 }
 

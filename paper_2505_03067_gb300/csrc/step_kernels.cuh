@@ -66,13 +66,14 @@ struct GuardBand {
 
 // One element of the fused preparation: flags, cell id, diffusivity factor
 // and c^n gathered from the lattice, then the row of every species.
+// R: the CTA's row products (not kTab).
 // kTab: the device-resident form (rows from the rate tables; tile coordinates
 // and tables written earlier in the same kernel, so read through L2).
 // gb (device-resident step): a tumour voxel in the guard band sets *hit.
 // kVar: the lattice has a diffusivity factor per voxel.
 template <bool kTab, bool kVar>
-__device__ __forceinline__ void prep_elem_t(const BatchSys &S, const BoxGeo &g, int64_t e, const RowTab *tab = nullptr,
-                                          const GuardBand *gb = nullptr, bool *hit = nullptr)
+__device__ __forceinline__ void prep_elem_t(const BatchSys &S, const BoxGeo &g, int64_t e, const RowCoef *R,
+                                            const RowTab *tab, const GuardBand *gb, bool *hit)
 {
     const int ns = S.C.nspecies;
     int bx, by, bz;
@@ -175,7 +176,7 @@ __device__ __forceinline__ void prep_elem_t(const BatchSys &S, const BoxGeo &g, 
             dg = dkv[s] + tab->aDn[s][__popc(f & F_OPEN) + 2 * ndir];
             bb = (c + dqv[s]) + tab->wbn[s][ndir];
         } else {
-            assemble_row(S.C, s, f, id, ndir, kVar, fp, hsum, c, dg, bb);
+            assemble_row(S.C, R, s, f, id, ndir, kVar, fp, hsum, c, dg, bb);
         }
         S.x[s][e] = c;
         S.cn[s][e] = c;
@@ -186,11 +187,12 @@ __device__ __forceinline__ void prep_elem_t(const BatchSys &S, const BoxGeo &g, 
 }
 
 template <bool kTab>
-__device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, int64_t e, const RowTab *tab = nullptr,
-                                          const GuardBand *gb = nullptr, bool *hit = nullptr)
+__device__ __forceinline__ void prep_elem(const BatchSys &S, const BoxGeo &g, int64_t e, const RowCoef *R = nullptr,
+                                          const RowTab *tab = nullptr, const GuardBand *gb = nullptr,
+                                          bool *hit = nullptr)
 {
-    if (S.dfac) prep_elem_t<kTab, true>(S, g, e, tab, gb, hit);
-    else prep_elem_t<kTab, false>(S, g, e, tab, gb, hit);
+    if (S.dfac) prep_elem_t<kTab, true>(S, g, e, R, tab, gb, hit);
+    else prep_elem_t<kTab, false>(S, g, e, R, tab, gb, hit);
 }
 
 // The device-resident preparation for uniform D on tiles at least four wide
@@ -509,8 +511,8 @@ __device__ __forceinline__ void gather_phase_t(const ExtractArgs &A, const Batch
         const int4 c = next;
         if (u + us < nunit) next = __ldcg(tcs + ((u + us) >> lu));
         if (chunks) prep_chunk<kAl>(S, g, (uint32_t)u, c, &tab, gb, &hit);
-        else if (VAR) prep_elem<true>(S, g, e, &tab, gb, &hit);
-        else prep_elem_t<true, false>(S, g, e, &tab, gb, &hit);
+        else if (VAR) prep_elem<true>(S, g, e, nullptr, &tab, gb, &hit);
+        else prep_elem_t<true, false>(S, g, e, nullptr, &tab, gb, &hit);
         if (nbr && (e & ((1 << ltv) - 1)) == 0) {   // neighbour tiles of this tile
             const int64_t a = e >> ltv;
 #pragma unroll
