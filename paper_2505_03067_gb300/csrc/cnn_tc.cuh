@@ -49,9 +49,7 @@ constexpr int kSlabX = 8, kSlabY = 16, kZSeg = 8;
 constexpr int kHaloX = kSlabX + 2, kHaloY = kSlabY + 2;
 // forward kernel: 12 epilogue warps, 6 loader warps and one warp that issues the
 // MMAs (19 warps, at most 5 on each SM sub-partition; 96 registers a thread).
-// With six loader warps a thread issues 7 halo copies per depth instead of
-// 11 with four, whose issue latency held the pipeline back (seven warps gain
-// nothing more, five less).
+// With six loader warps a thread issues three halo copies per depth.
 constexpr int kEpiWarps = 12, kLoadWarps = 6;
 constexpr int kConvThreads = 32 * (kEpiWarps + kLoadWarps + 1);
 constexpr int kFwdSlots = 10;           // halo depths in the forward kernel's ring
@@ -381,8 +379,8 @@ __device__ __forceinline__ bool in_box(const CnnDom &D, int b, int x, int y, int
            z >= D.lo[b][2] && z < D.lo[b][2] + D.n[b][2];
 }
 
-// The 16-byte copies of one halo depth handled by one loader thread, fixed for
-// a launch: the k-th covers item tid + k NL of the depth (halo row yh, copy c,
+// Weight gradient: the 16-byte copies of one halo depth handled by one loader
+// thread, fixed for a launch: the k-th covers item tid + k NL of the depth (halo row yh, copy c,
 // channel chunk kc, x row; x fastest, so the eight lanes that fill one core
 // matrix write its 128 contiguous bytes -- one shared-memory wavefront, no
 // bank conflict -- while a warp still reads the same sectors of the source
