@@ -561,12 +561,16 @@ mpm_status mpm_scatter(mpm_ctx *ctx, const mpm_subgrid *sub, const mpm_lattice *
  *  MPM_DEBUG_CNN_LAYER_TIMES 1: every later network application outside a
  *                        graph capture records CUDA events around each of its
  *                        six convolution launches (read with
- *                        mpm_cnn_layer_times). */
+ *                        mpm_cnn_layer_times).
+ *  MPM_DEBUG_REFUSE_ALLOC  n: the context's n-th request for device memory from
+ *                        now on (mpm_create's aside) is refused as on a full
+ *                        device (0 = none, the default). */
 #define MPM_DEBUG_TIMEOUT_NS 1
 #define MPM_DEBUG_SKIP_BLOCK 2
 #define MPM_DEBUG_PHASE_TIMES 3
 #define MPM_DEBUG_SOLVER_VARIANT 4
 #define MPM_DEBUG_CNN_LAYER_TIMES 5
+#define MPM_DEBUG_REFUSE_ALLOC 6
 mpm_status mpm_debug_set(mpm_ctx *ctx, int32_t key, int64_t value);
 
 /* Test hook: the FP32 Krylov path's bit-level conversions applied to n
@@ -621,6 +625,9 @@ mpm_status mpm_debug_convert(const double *in64, float *out32, float *ref32, con
  * step's graph was last set up, as of the last step waited for (with
  * mpm_opts.box_every > 1 the other steps keep the box). */
 #define MPM_COUNTER_STEP_FULL_EXTRACTIONS 19
+/* Device memory that the context's subgrids hold for the means of a per-voxel
+ * diffusivity across the faces (mpm_step). */
+#define MPM_COUNTER_FACE_MEANS_BYTES 20
 mpm_status mpm_counter_get(const mpm_ctx *ctx, int32_t key, int64_t *value);
 
 /*

@@ -22,6 +22,22 @@ mpm_status mpm_cuda_check(mpm_ctx *ctx, cudaError_t e, const char *what)
     return mpm_fail(ctx, MPM_ERR_CUDA, m);
 }
 
+// cudaMalloc for the context.  A refused request leaves no error behind in the
+// runtime: the next launch check would take it for its own.  (refuse_alloc:
+// test hook, the request that many calls from now asks for 64 TiB instead, more
+// than any device holds.)
+static cudaError_t try_malloc(mpm_ctx *ctx, void **q, size_t bytes)
+{
+    const bool refuse = ctx->refuse_alloc > 0 && --ctx->refuse_alloc == 0;
+    *q = nullptr;
+    const cudaError_t e = cudaMalloc(q, refuse ? (size_t)1 << 46 : bytes);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *q = nullptr;
+    }
+    return e;
+}
+
 // Grow-only device buffer under the context's cap; the old contents are not kept.
 mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char *what)
 {
@@ -40,15 +56,13 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
         *cap = 0;
     }
     void *q = nullptr;
-    cudaError_t e = cudaMalloc(&q, want);
+    cudaError_t e = try_malloc(ctx, &q, want);
     if (e == cudaErrorMemoryAllocation && !ctx->hm_subs.empty()) {   // the face means are optional: give them up
         while (!ctx->hm_subs.empty()) mpm_face_means_free(ctx, ctx->hm_subs.back());
-        e = cudaMalloc(&q, want);
+        e = try_malloc(ctx, &q, want);
     }
-    if (e != cudaSuccess) {
-        cudaGetLastError();
+    if (e != cudaSuccess)
         return mpm_fail(ctx, MPM_ERR_NOMEM, std::string(what) + ": cudaMalloc of " + std::to_string(want) + " bytes failed");
-    }
     *p = q;
     *cap = want;
     ctx->allocated += want;
@@ -71,12 +85,9 @@ void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n)
     if (6 * stride > sub->hm_cap) {
         mpm_face_means_free(ctx, sub);
         const int64_t want = 6 * (stride + stride / 4);
-        double *q = nullptr;
-        if (cudaMalloc(&q, (size_t)want * sizeof(double)) != cudaSuccess) {
-            cudaGetLastError();
-            return;
-        }
-        sub->hm = q;
+        void *q = nullptr;
+        if (try_malloc(ctx, &q, (size_t)want * sizeof(double)) != cudaSuccess) return;
+        sub->hm = (double *)q;
         sub->hm_cap = want;
         ctx->allocated += (size_t)want * sizeof(double);
         ctx->hm_subs.push_back(sub);
@@ -469,6 +480,10 @@ mpm_status mpm_debug_set(mpm_ctx *ctx, int32_t key, int64_t value)
     case MPM_DEBUG_CNN_LAYER_TIMES:
         ctx->cnn_layer_prof = value != 0;
         return MPM_OK;
+    case MPM_DEBUG_REFUSE_ALLOC:
+        if (value < 0) return mpm_fail(ctx, MPM_ERR_ARG, "debug: negative allocation index");
+        ctx->refuse_alloc = value;
+        return MPM_OK;
     default:
         return mpm_fail(ctx, MPM_ERR_ARG, "debug: unknown key");
     }
@@ -511,6 +526,11 @@ mpm_status mpm_counter_get(const mpm_ctx *ctx, int32_t key, int64_t *value)
         return MPM_OK;
     }
     if (key == MPM_COUNTER_STEP_FULL_EXTRACTIONS) { *value = ctx->step_nfull; return MPM_OK; }
+    if (key == MPM_COUNTER_FACE_MEANS_BYTES) {
+        *value = 0;
+        for (const mpm_subgrid *s : ctx->hm_subs) *value += s->hm_cap * (int64_t)sizeof(double);
+        return MPM_OK;
+    }
     return MPM_ERR_ARG;
 }
 

@@ -485,6 +485,7 @@ struct mpm_ctx {
     // test hooks
     uint64_t timeout_ns = 2000000000ull;
     int32_t skip_block = -1;
+    int64_t refuse_alloc = 0;    // the device allocation that many requests from now is refused (0: none)
 };
 
 struct mpm_subgrid {

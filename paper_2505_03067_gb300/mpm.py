@@ -19,7 +19,8 @@ OK, ERR_ARG, ERR_EMPTY, ERR_NOCONV, ERR_BREAKDOWN, ERR_TIMEOUT, ERR_CUDA, ERR_NO
 STATUS_NAMES = ["OK", "ERR_ARG", "ERR_EMPTY", "ERR_NOCONV", "ERR_BREAKDOWN", "ERR_TIMEOUT", "ERR_CUDA", "ERR_NOMEM"]
 EXPORT_X, EXPORT_RHS, EXPORT_DIAG, EXPORT_FLAGS, EXPORT_CELL = range(5)
 DEBUG_TIMEOUT_NS, DEBUG_SKIP_BLOCK, DEBUG_PHASE_TIMES, DEBUG_SOLVER_VARIANT, DEBUG_CNN_LAYER_TIMES = 1, 2, 3, 4, 5
-COUNTER_STEP_FULL_EXTRACTIONS = 19
+DEBUG_REFUSE_ALLOC = 6
+COUNTER_STEP_FULL_EXTRACTIONS, COUNTER_FACE_MEANS_BYTES = 19, 20
 CNN_INPUT, CNN_TARGET = 0, 1
 
 _HERE = os.path.dirname(os.path.abspath(__file__))

@@ -1,0 +1,76 @@
+"""Memory of the stored face means of a per-voxel diffusivity: they are optional
+and given up when the device is full, and nothing else depends on them.  A
+refused device allocation is made by the test hook; every system must come out
+at the oracle's step (the bound is that of test_gpu_face_means.py: the residual
+is driven to TOL, and A is an M-matrix with smallest eigenvalue >= 1)."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2505_03067_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-13
+BOUND = 1e-10
+
+
+@pytest.fixture(scope="module")
+def M():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2505_03067_gb300 import build, mpm
+    build.build()
+    return mpm
+
+
+@pytest.fixture(scope="module")
+def case():
+    wl = W.random_case(31, (21, 13, 11), nspecies=3, dfac=True)
+    ref, states = wl.lattice.copy(), []
+    for _ in range(3):
+        oracle.step(ref, wl.params, wl.margin, rtol=0.0, atol=TOL)
+        states.append(ref.fields.copy())
+    return wl, states
+
+
+class System:
+    """One subgrid of ctx on a lattice of its own, stepped in one of three forms."""
+
+    def __init__(self, M, ctx, wl, form):
+        self.M, self.n = M, 0
+        self.lat, self.prm = M.DeviceLattice(wl.lattice), M.DeviceParams(wl.params)
+        if form == "batch":
+            self.b = M.BatchStepper(ctx, [self.lat], [self.prm], [wl.margin])
+            self.sub, self._step = self.b.subs[0], lambda o: self.b.step(o)[0]
+        else:
+            s = M.StepSolver(ctx, self.lat, self.prm, wl.margin, fused=form == "step")
+            self.sub, self._step = s.sub, lambda o: s.step(o)["status_code"]
+
+    def step(self, restart=16):
+        opts = self.M.make_opts(rtol=0.0, atol=TOL, restart=restart, maxit=800)
+        assert self._step(opts) == self.M.OK
+        self.n += 1
+
+    def error(self, states):
+        return np.max(np.abs(self.lat.fields_numpy() - states[self.n - 1]))
+
+
+def held(M, ctx):
+    return ctx.counter(M.COUNTER_FACE_MEANS_BYTES)
+
+
+@pytest.mark.parametrize("form", ["composed", "step", "batch"])
+def test_a_call_that_had_to_give_the_means_up_succeeds(M, case, form):
+    wl, states = case
+    ctx = M.Context(0)
+    a = System(M, ctx, wl, form)
+    a.step()
+    assert held(M, ctx) > 0
+    ctx.debug_set(M.DEBUG_REFUSE_ALLOC, 1)
+    b = System(M, ctx, wl, form)
+    b.step()
+    a.step()
+    b.step()
+    assert a.error(states) <= BOUND and b.error(states) <= BOUND
