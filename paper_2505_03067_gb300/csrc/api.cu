@@ -38,6 +38,19 @@ static cudaError_t try_malloc(mpm_ctx *ctx, void **q, size_t bytes)
     return e;
 }
 
+// Device memory of the context (*q = nullptr when there is none).  Every buffer
+// but the face means comes from here: those are optional (mpm_face_means), so on
+// a full device they are given up and the request is made once more.
+cudaError_t mpm_dev_malloc(mpm_ctx *ctx, void **q, size_t bytes)
+{
+    cudaError_t e = try_malloc(ctx, q, bytes);
+    if (e == cudaErrorMemoryAllocation && !ctx->hm_subs.empty()) {
+        while (!ctx->hm_subs.empty()) mpm_face_means_free(ctx, ctx->hm_subs.back());
+        e = try_malloc(ctx, q, bytes);
+    }
+    return e;
+}
+
 // Grow-only device buffer under the context's cap; the old contents are not kept.
 mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char *what)
 {
@@ -56,12 +69,7 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
         *cap = 0;
     }
     void *q = nullptr;
-    cudaError_t e = try_malloc(ctx, &q, want);
-    if (e == cudaErrorMemoryAllocation && !ctx->hm_subs.empty()) {   // the face means are optional: give them up
-        while (!ctx->hm_subs.empty()) mpm_face_means_free(ctx, ctx->hm_subs.back());
-        e = try_malloc(ctx, &q, want);
-    }
-    if (e != cudaSuccess)
+    if (mpm_dev_malloc(ctx, &q, want) != cudaSuccess)
         return mpm_fail(ctx, MPM_ERR_NOMEM, std::string(what) + ": cudaMalloc of " + std::to_string(want) + " bytes failed");
     *p = q;
     *cap = want;

@@ -716,12 +716,8 @@ namespace {
 
 mpm_status cnn_alloc(mpm_ctx *ctx, mpm_cnn *c, void **p, size_t bytes)
 {
-    cudaError_t e = cudaMalloc(p, bytes ? bytes : 16);
-    if (e != cudaSuccess) {
-        cudaGetLastError();
-        *p = nullptr;
+    if (mpm_dev_malloc(ctx, p, bytes ? bytes : 16) != cudaSuccess)
         return mpm_fail(ctx, MPM_ERR_NOMEM, "cnn: device allocation failed");
-    }
     c->allocs.push_back(*p);
     return MPM_OK;
 }

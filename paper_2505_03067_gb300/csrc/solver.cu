@@ -538,10 +538,10 @@ mpm_status mpm_solve_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm_latt
         if (ctx->d_bar) cudaFree(ctx->d_bar);
         ctx->d_bar = nullptr;
         ctx->bar_cap = 0;
-        MPM_CU(cudaMalloc(&ctx->d_bar, (size_t)P.nteam * 32 * sizeof(uint32_t)));
+        MPM_CU(mpm_dev_malloc(ctx, (void **)&ctx->d_bar, (size_t)P.nteam * 32 * sizeof(uint32_t)));
         ctx->bar_cap = P.nteam;
     }
-    if (ctx->phase_prof && !ctx->d_prof) MPM_CU(cudaMalloc(&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
+    if (ctx->phase_prof && !ctx->d_prof) MPM_CU(mpm_dev_malloc(ctx, (void **)&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
     // the staging buffer is free: every call that uses it ends with a stream synchronisation
     char *hs = (char *)ctx->h_stage;
     fill_descriptors(P, subs, hs);
@@ -668,8 +668,8 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
         if (r != MPM_OK) return r;
         B->plan.sa.partials = B->d_partials;
         if (!B->d_bar) {
-            MPM_CU(cudaMalloc(&B->d_bar, (size_t)ctx->num_sms * 4 * 32 * sizeof(uint32_t)));
-            MPM_CU(cudaMalloc(&B->d_abort, 256));
+            MPM_CU(mpm_dev_malloc(ctx, (void **)&B->d_bar, (size_t)ctx->num_sms * 4 * 32 * sizeof(uint32_t)));
+            MPM_CU(mpm_dev_malloc(ctx, (void **)&B->d_abort, 256));
         }
         if (B->plan.nteam > ctx->num_sms * 4) return mpm_fail(ctx, MPM_ERR_ARG, "batch_step: too many teams");
         r = ensure_stage(ctx, B->plan.args_need + 4096);
@@ -722,7 +722,7 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
         // eager form of the same sequence (graph unavailable or phase timing on)
         r = mpm_batch_prep_launch(ctx, B->d_desc, nsys, B->prep_blocks, var, st);
         if (r != MPM_OK) return r;
-        if (ctx->phase_prof && !ctx->d_prof) MPM_CU(cudaMalloc(&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
+        if (ctx->phase_prof && !ctx->d_prof) MPM_CU(mpm_dev_malloc(ctx, (void **)&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
         r = enqueue_solve(ctx, P, B->d_args, B->d_bar, B->d_abort, ctx->phase_prof ? ctx->d_prof : nullptr, st);
         if (r != MPM_OK) return r;
         r = mpm_batch_scatter_launch(ctx, B->d_desc, nsys, B->prep_blocks, st);
@@ -996,9 +996,9 @@ mpm_status mpm_step_enqueue_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_latti
     int G = opt->nblocks > 0 ? std::min(opt->nblocks, gmax) : step_grid(NE_est, S, gmax, var.nt);
     if (opt->nblocks <= 0 && T->G > 0 && T->G <= gmax && G >= T->G * 4 / 5 && G <= T->G * 5 / 4) G = T->G;
     if (!T->d_scr) {
-        MPM_CU(cudaMalloc(&T->d_scr, 1024));
+        MPM_CU(mpm_dev_malloc(ctx, (void **)&T->d_scr, 1024));
         MPM_CU(cudaMemset(T->d_scr, 0, 1024));
-        MPM_CU(cudaMalloc(&T->d_bar, (size_t)ctx->num_sms * 4 * 32 * sizeof(uint32_t)));
+        MPM_CU(mpm_dev_malloc(ctx, (void **)&T->d_bar, (size_t)ctx->num_sms * 4 * 32 * sizeof(uint32_t)));
         T->valid = false;
     }
     auto make_key = [&](std::vector<unsigned char> &key) {
@@ -1062,7 +1062,7 @@ mpm_status mpm_step_enqueue_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_latti
             T->hout_cap = hneed;
             MPM_CU(cudaHostGetDevicePointer((void **)&T->h_out_dev, T->h_out, 0));
         }
-        if (ctx->phase_prof && !ctx->d_prof) MPM_CU(cudaMalloc(&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
+        if (ctx->phase_prof && !ctx->d_prof) MPM_CU(mpm_dev_malloc(ctx, (void **)&ctx->d_prof, kProfSlots * sizeof(unsigned long long)));
         r = ensure_stage(ctx, T->plan.args_need + 4096);
         if (r != MPM_OK) return r;
         fill_descriptors(T->plan, &sub, (char *)ctx->h_stage);

@@ -74,3 +74,33 @@ def test_a_call_that_had_to_give_the_means_up_succeeds(M, case, form):
     a.step()
     b.step()
     assert a.error(states) <= BOUND and b.error(states) <= BOUND
+
+
+@pytest.mark.parametrize("form", ["composed", "step", "batch"])
+def test_whichever_allocation_is_refused_the_call_succeeds(M, case, form):
+    """A second subgrid makes at most ten device allocations of its own (the
+    device-resident step: tile tables, elements, means, scratch, barriers, Krylov
+    bases, descriptors, partials, rates, extraction scratch)."""
+    wl, states = case
+    for n in range(1, 12):
+        ctx = M.Context(0)
+        a = System(M, ctx, wl, form)
+        a.step()
+        ctx.debug_set(M.DEBUG_REFUSE_ALLOC, n)
+        b = System(M, ctx, wl, form)
+        b.step()
+        assert a.error(states) <= BOUND and b.error(states) <= BOUND, n
+        a.step()
+        assert a.error(states) <= BOUND, n
+
+
+def test_a_network_takes_the_memory_of_the_means(M, case):
+    wl, states = case
+    ctx = M.Context(0)
+    a = System(M, ctx, wl, "step")
+    a.step()
+    ctx.debug_set(M.DEBUG_REFUSE_ALLOC, 1)
+    M.CNN(ctx, wl.lattice.dims, 1, M.cnn_init_params(1))
+    assert held(M, ctx) == 0
+    a.step()
+    assert a.error(states) <= BOUND
