@@ -83,7 +83,8 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
 // a pass had six per element).  They are not counted as workspace the caller
 // must provide: a context with a memory cap goes without them, as does one
 // whose device is full, and the solver then forms the means in every pass.
-void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n)
+// room >= n: the elements that a new buffer is made for.
+void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room)
 {
     if (!sub->has_dfac || ctx->cap || n < 1) {
         mpm_face_means_free(ctx, sub);
@@ -92,7 +93,7 @@ void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n)
     const int64_t stride = (n + 31) & ~(int64_t)31;
     if (6 * stride > sub->hm_cap) {
         mpm_face_means_free(ctx, sub);
-        const int64_t want = 6 * (stride + stride / 4);
+        const int64_t want = 6 * ((room + 31) & ~(int64_t)31);
         void *q = nullptr;
         if (try_malloc(ctx, &q, (size_t)want * sizeof(double)) != cudaSuccess) return;
         sub->hm = (double *)q;

@@ -797,7 +797,7 @@ mpm_status mpm_step_buffers(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_lattice *l
     sub->nspecies = nspecies;
     sub->has_dfac = has_dfac;
     sub->NE_cap = (int64_t)NE;
-    mpm_face_means(ctx, sub, (int64_t)NE);
+    mpm_face_means(ctx, sub, (int64_t)NE, (int64_t)NE);
     return MPM_OK;
 }
 

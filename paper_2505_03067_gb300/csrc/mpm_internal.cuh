@@ -540,7 +540,7 @@ mpm_status mpm_fail(mpm_ctx *ctx, mpm_status st, const std::string &msg);
 mpm_status mpm_cuda_check(mpm_ctx *ctx, cudaError_t e, const char *what);
 cudaError_t mpm_dev_malloc(mpm_ctx *ctx, void **q, size_t bytes);
 mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char *what);
-void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n);   // room for the face means of n elements, if any
+void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room);   // a place for the face means of n elements, if any
 void mpm_face_means_free(mpm_ctx *ctx, mpm_subgrid *sub);
 
 #define MPM_CU(call)                                                       \

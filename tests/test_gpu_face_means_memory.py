@@ -104,3 +104,10 @@ def test_a_network_takes_the_memory_of_the_means(M, case):
     assert held(M, ctx) == 0
     a.step()
     assert a.error(states) <= BOUND
+
+
+def test_the_step_holds_48_bytes_a_stored_voxel(M, case):
+    wl, _ = case
+    ctx = M.Context(0)
+    System(M, ctx, wl, "step").step()
+    assert held(M, ctx) == 48 * 24 * 16 * 12      # the lattice of 21 x 13 x 11 in tiles of 4 x 4 x 4
