@@ -83,6 +83,10 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
 // a pass had six per element).  They are not counted as workspace the caller
 // must provide: a context with a memory cap goes without them, as does one
 // whose device is full, and the solver then forms the means in every pass.
+// Called where the element buffers are made (extraction, device-resident step)
+// and nowhere else: whoever uses the subgrid later may be recording a CUDA graph
+// (the assembly allocates nothing), and a buffer made after the assembly would
+// hold no means.
 // room >= n: the elements that a new buffer is made for.
 void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room)
 {

@@ -173,7 +173,6 @@ mpm_status mpm_assemble_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_params *p
     A.flags = sub->flags;
     A.cell = sub->cell;
     A.dfac = sub->dfac;
-    mpm_face_means(ctx, sub, sub->NE, sub->NE + sub->NE / 4);   // head-room for growing boxes, as mpm_grow's
     A.hm = sub->hm;
     A.hstride = sub->hm_stride;
     A.tile_coord = sub->tile_coord;

@@ -544,6 +544,7 @@ mpm_status mpm_extract_impl(mpm_ctx *ctx, const mpm_lattice *lat, int32_t nspeci
     tmp.assembled = false;
     tmp.x_fresh = true;
     *sub = tmp;
+    mpm_face_means(ctx, sub, sub->NE, sub->NE + sub->NE / 4);   // head-room for growing boxes, as mpm_grow's
     if (out_box) *out_box = box;
     return MPM_OK;
 }

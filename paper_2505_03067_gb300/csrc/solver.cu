@@ -637,10 +637,7 @@ mpm_status mpm_batch_step_impl(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm
     if (!ctx->batch_graph) ctx->batch_graph = new BatchGraph();
     BatchGraph *B = (BatchGraph *)ctx->batch_graph;
     bool var = false;   // part of the key: gen changes with the extraction, and dfac's presence with it
-    for (int i = 0; i < nsys; ++i) {
-        mpm_face_means(ctx, subs[i], subs[i]->NE, subs[i]->NE);
-        var |= subs[i]->has_dfac;
-    }
+    for (int i = 0; i < nsys; ++i) var |= subs[i]->has_dfac;
     std::vector<unsigned char> key;
     batch_key(ctx, subs, lats, prms, nsys, opt, key);
     const bool use_graph = !ctx->phase_prof;

@@ -111,3 +111,37 @@ def test_the_step_holds_48_bytes_a_stored_voxel(M, case):
     ctx = M.Context(0)
     System(M, ctx, wl, "step").step()
     assert held(M, ctx) == 48 * 24 * 16 * 12      # the lattice of 21 x 13 x 11 in tiles of 4 x 4 x 4
+
+
+def test_a_batch_makes_no_means_of_its_own(M, case):
+    """Given up while the batch is planned again, the means stay given up until
+    the next extraction: a buffer of a later call would not have been filled."""
+    wl, states = case
+    ctx = M.Context(0)
+    a = System(M, ctx, wl, "batch")
+    a.step(8)
+    assert held(M, ctx) > 0
+    ctx.debug_set(M.DEBUG_REFUSE_ALLOC, 1)
+    a.step(32)                                    # longer restart: the Krylov bases grow
+    assert held(M, ctx) == 0
+    a.step(32)
+    assert held(M, ctx) == 0 and a.error(states) <= BOUND
+
+
+def test_refresh_and_assembly_can_be_captured(M, case):
+    import torch
+    wl, states = case
+    ctx = M.Context(0)
+    System(M, ctx, wl, "composed").step()         # every kernel is loaded
+    lat, prm, sub = M.DeviceLattice(wl.lattice), M.DeviceParams(wl.params), ctx.subgrid_create()
+    sub.mpm_box_extract(lat, 3, wl.margin)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        sub.mpm_subgrid_refresh(lat)
+        sub.mpm_assemble_coeffs(prm)
+    opts = M.make_opts(rtol=0.0, atol=TOL, restart=16, maxit=800)
+    for want in states:
+        g.replay()
+        sub.mpm_solve_step(opts, scatter_to=lat)
+        assert np.max(np.abs(lat.fields_numpy() - want)) <= BOUND
