@@ -45,7 +45,11 @@ cudaError_t mpm_dev_malloc(mpm_ctx *ctx, void **q, size_t bytes)
 {
     cudaError_t e = try_malloc(ctx, q, bytes);
     if (e == cudaErrorMemoryAllocation && !ctx->hm_subs.empty()) {
-        while (!ctx->hm_subs.empty()) mpm_face_means_free(ctx, ctx->hm_subs.back());
+        while (!ctx->hm_subs.empty()) {
+            mpm_subgrid *sub = ctx->hm_subs.back();
+            sub->hm_refused = sub->hm_cap;
+            mpm_face_means_free(ctx, sub);
+        }
         e = try_malloc(ctx, q, bytes);
     }
     return e;
@@ -86,7 +90,9 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
 // Called where the element buffers are made (extraction, device-resident step)
 // and nowhere else: whoever uses the subgrid later may be recording a CUDA graph
 // (the assembly allocates nothing), and a buffer made after the assembly would
-// hold no means.
+// hold no means.  A size that the device once had no room for is not requested
+// again for the subgrid: the device-resident step comes here every time, and
+// would pay for a refused request every time.
 // room >= n: the elements that a new buffer is made for.
 void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room)
 {
@@ -98,8 +104,12 @@ void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room)
     if (6 * stride > sub->hm_cap) {
         mpm_face_means_free(ctx, sub);
         const int64_t want = 6 * ((room + 31) & ~(int64_t)31);
+        if (sub->hm_refused && want >= sub->hm_refused) return;
         void *q = nullptr;
-        if (try_malloc(ctx, &q, (size_t)want * sizeof(double)) != cudaSuccess) return;
+        if (try_malloc(ctx, &q, (size_t)want * sizeof(double)) != cudaSuccess) {
+            sub->hm_refused = want;
+            return;
+        }
         sub->hm = (double *)q;
         sub->hm_cap = want;
         ctx->allocated += (size_t)want * sizeof(double);

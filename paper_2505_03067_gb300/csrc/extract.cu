@@ -539,6 +539,7 @@ mpm_status mpm_extract_impl(mpm_ctx *ctx, const mpm_lattice *lat, int32_t nspeci
     tmp.hm = sub->hm;   // allocating the buffers above may have given them up
     tmp.hm_stride = sub->hm_stride;
     tmp.hm_cap = sub->hm_cap;
+    tmp.hm_refused = sub->hm_refused;
     tmp.gen = sub->gen + 1;
     tmp.extracted = true;
     tmp.assembled = false;

@@ -521,6 +521,7 @@ struct mpm_subgrid {
     // solver forms them in every pass
     double *hm = nullptr;
     int64_t hm_stride = 0, hm_cap = 0;   // doubles per face, doubles allocated
+    int64_t hm_refused = 0;              // doubles the device had no room for (0: not so far)
     double *x[MPM_MAX_SPECIES] = {};
     double *cn[MPM_MAX_SPECIES] = {};
     double *b[MPM_MAX_SPECIES] = {};

@@ -145,3 +145,18 @@ def test_refresh_and_assembly_can_be_captured(M, case):
         g.replay()
         sub.mpm_solve_step(opts, scatter_to=lat)
         assert np.max(np.abs(lat.fields_numpy() - want)) <= BOUND
+
+
+@pytest.mark.parametrize("form", ["composed", "step"])
+@pytest.mark.parametrize("nth", [1, 3])           # the next growing buffer; the means' own request
+def test_means_without_room_are_not_requested_again(M, case, form, nth):
+    wl, states = case
+    ctx = M.Context(0)
+    a = System(M, ctx, wl, form)
+    if nth == 1:
+        a.step(8)
+    ctx.debug_set(M.DEBUG_REFUSE_ALLOC, nth)
+    a.step(32)                                    # tile tables, elements, means; Krylov bases
+    assert held(M, ctx) == 0
+    a.step(32)
+    assert held(M, ctx) == 0 and a.error(states) <= BOUND
