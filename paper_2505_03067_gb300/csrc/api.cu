@@ -5,6 +5,7 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
+#include <vector>
 
 #include "mpm_internal.cuh"
 
@@ -43,16 +44,17 @@ static cudaError_t try_malloc(mpm_ctx *ctx, void **q, size_t bytes)
 // a full device they are given up and the request is made once more.
 cudaError_t mpm_dev_malloc(mpm_ctx *ctx, void **q, size_t bytes)
 {
-    cudaError_t e = try_malloc(ctx, q, bytes);
-    if (e == cudaErrorMemoryAllocation && !ctx->hm_subs.empty()) {
-        while (!ctx->hm_subs.empty()) {
-            mpm_subgrid *sub = ctx->hm_subs.back();
-            sub->hm_refused = sub->hm_cap;
-            mpm_face_means_free(ctx, sub);
-        }
-        e = try_malloc(ctx, q, bytes);
+    const cudaError_t e = try_malloc(ctx, q, bytes);
+    if (e != cudaErrorMemoryAllocation) return e;
+    std::vector<mpm_subgrid *> subs;
+    for (mpm_subgrid *sub : ctx->hm_subs)
+        if (!sub->hm_recorded) subs.push_back(sub);
+    if (subs.empty()) return e;
+    for (mpm_subgrid *sub : subs) {
+        sub->hm_refused = sub->hm_cap;
+        mpm_face_means_free(ctx, sub);
     }
-    return e;
+    return try_malloc(ctx, q, bytes);
 }
 
 // Grow-only device buffer under the context's cap; the old contents are not kept.
@@ -118,10 +120,23 @@ void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room)
     sub->hm_stride = stride;
 }
 
+// A caller's graph that records an assembly or a step holds the means' address
+// and may be replayed as long as the subgrid's own buffers stand: from then on
+// the buffer is neither given up nor freed before the subgrid is.
+void mpm_face_means_record(mpm_subgrid *sub, cudaStream_t st)
+{
+    if (!sub->hm || sub->hm_recorded) return;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) cudaGetLastError();   // the legacy stream beside a capture
+    else if (cs != cudaStreamCaptureStatusNone) sub->hm_recorded = true;
+}
+
 void mpm_face_means_free(mpm_ctx *ctx, mpm_subgrid *sub)
 {
     if (!sub->hm) return;
-    cudaFree(sub->hm);
+    if (sub->hm_recorded) sub->hm_kept.push_back(sub->hm);
+    else cudaFree(sub->hm);
+    sub->hm_recorded = false;
     if (ctx) {
         ctx->allocated -= (size_t)sub->hm_cap * sizeof(double);
         ctx->hm_subs.erase(std::remove(ctx->hm_subs.begin(), ctx->hm_subs.end(), sub), ctx->hm_subs.end());
@@ -134,6 +149,8 @@ static void free_sub_buffers(mpm_ctx *ctx, mpm_subgrid *sub)
 {
     mpm_step_free(ctx, sub);
     mpm_face_means_free(ctx, sub);
+    for (double *p : sub->hm_kept) cudaFree(p);
+    sub->hm_kept.clear();
     void **bufs[3] = {&sub->geo, &sub->elem, &sub->krylov};
     size_t *caps[3] = {&sub->geo_bytes, &sub->elem_bytes, &sub->krylov_bytes};
     for (int i = 0; i < 3; ++i) {

@@ -173,6 +173,7 @@ mpm_status mpm_assemble_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_params *p
     A.flags = sub->flags;
     A.cell = sub->cell;
     A.dfac = sub->dfac;
+    mpm_face_means_record(sub, st);
     A.hm = sub->hm;
     A.hstride = sub->hm_stride;
     A.tile_coord = sub->tile_coord;

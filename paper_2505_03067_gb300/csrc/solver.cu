@@ -974,6 +974,7 @@ mpm_status mpm_step_enqueue_impl(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_latti
     r = mpm_step_buffers(ctx, sub, lat, S, lt);
     if (r != MPM_OK) return r;
     if (sub->geo != old_geo || sub->elem != old_elem) T->valid = false;
+    mpm_face_means_record(sub, st);
     // grid: from the previous step's element count, kept while within 25%;
     // at most the co-resident CTAs of the whole-step kernel
     const int maxm = opt->restart <= 8 ? 8 : (opt->restart <= 16 ? 16 : 32);

@@ -160,3 +160,30 @@ def test_means_without_room_are_not_requested_again(M, case, form, nth):
     assert held(M, ctx) == 0
     a.step(32)
     assert held(M, ctx) == 0 and a.error(states) <= BOUND
+
+
+def test_means_that_a_recorded_graph_writes_stay(M, case):
+    import torch
+    wl, states = case
+    System(M, M.Context(0), wl, "composed").step()     # every kernel is loaded
+    ctx = M.Context(0)
+    lat, prm, sub = M.DeviceLattice(wl.lattice), M.DeviceParams(wl.params), ctx.subgrid_create()
+    sub.mpm_box_extract(lat, 3, wl.margin)
+    before = held(M, ctx)
+    g = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(g):
+        sub.mpm_subgrid_refresh(lat)
+        sub.mpm_assemble_coeffs(prm)
+    ctx.debug_set(M.DEBUG_REFUSE_ALLOC, 1)
+    with pytest.raises(M.MpmError):                    # nothing that could be given up
+        M.CNN(ctx, wl.lattice.dims, 1, M.cnn_init_params(1))
+    assert held(M, ctx) == before > 0
+    opts = M.make_opts(rtol=0.0, atol=TOL, restart=16, maxit=800)
+    for want in states:
+        g.replay()
+        sub.mpm_solve_step(opts, scatter_to=lat)
+        assert np.max(np.abs(lat.fields_numpy() - want)) <= BOUND
+    uniform = M.DeviceLattice(W.random_case(31, (21, 13, 11), nspecies=3).lattice)
+    sub.mpm_box_extract(uniform, 3, wl.margin)         # leaves the buffer to the graph
+    assert held(M, ctx) == 0
