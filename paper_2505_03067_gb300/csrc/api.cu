@@ -52,7 +52,7 @@ cudaError_t mpm_dev_malloc(mpm_ctx *ctx, void **q, size_t bytes)
     if (subs.empty()) return e;
     for (mpm_subgrid *sub : subs) {
         sub->hm_refused = sub->hm_cap;
-        mpm_face_means_free(ctx, sub);
+        mpm_face_means_free(sub);
     }
     return try_malloc(ctx, q, bytes);
 }
@@ -99,12 +99,13 @@ mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char
 void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room)
 {
     if (!sub->has_dfac || ctx->cap || n < 1) {
-        mpm_face_means_free(ctx, sub);
+        mpm_face_means_free(sub);
         return;
     }
+    if (sub->hm_ctx != ctx) mpm_face_means_free(sub);   // the context that uses them accounts for them
     const int64_t stride = (n + 31) & ~(int64_t)31;
     if (6 * stride > sub->hm_cap) {
-        mpm_face_means_free(ctx, sub);
+        mpm_face_means_free(sub);
         const int64_t want = 6 * ((room + 31) & ~(int64_t)31);
         if (sub->hm_refused && want >= sub->hm_refused) return;
         void *q = nullptr;
@@ -114,6 +115,7 @@ void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room)
         }
         sub->hm = (double *)q;
         sub->hm_cap = want;
+        sub->hm_ctx = ctx;
         ctx->allocated += (size_t)want * sizeof(double);
         ctx->hm_subs.push_back(sub);
     }
@@ -131,24 +133,25 @@ void mpm_face_means_record(mpm_subgrid *sub, cudaStream_t st)
     else if (cs != cudaStreamCaptureStatusNone) sub->hm_recorded = true;
 }
 
-void mpm_face_means_free(mpm_ctx *ctx, mpm_subgrid *sub)
+void mpm_face_means_free(mpm_subgrid *sub)
 {
     if (!sub->hm) return;
     if (sub->hm_recorded) sub->hm_kept.push_back(sub->hm);
     else cudaFree(sub->hm);
     sub->hm_recorded = false;
-    if (ctx) {
+    if (mpm_ctx *ctx = sub->hm_ctx) {
         ctx->allocated -= (size_t)sub->hm_cap * sizeof(double);
         ctx->hm_subs.erase(std::remove(ctx->hm_subs.begin(), ctx->hm_subs.end(), sub), ctx->hm_subs.end());
     }
     sub->hm = nullptr;
+    sub->hm_ctx = nullptr;
     sub->hm_stride = sub->hm_cap = 0;
 }
 
 static void free_sub_buffers(mpm_ctx *ctx, mpm_subgrid *sub)
 {
     mpm_step_free(ctx, sub);
-    mpm_face_means_free(ctx, sub);
+    mpm_face_means_free(sub);
     for (double *p : sub->hm_kept) cudaFree(p);
     sub->hm_kept.clear();
     void **bufs[3] = {&sub->geo, &sub->elem, &sub->krylov};
@@ -244,6 +247,7 @@ mpm_status mpm_destroy(mpm_ctx *ctx)
     if (!ctx) return MPM_ERR_ARG;
     mpm_batch_graph_free(ctx);
     mpm_fgmres_release(ctx);
+    for (mpm_subgrid *sub : ctx->hm_subs) sub->hm_ctx = nullptr;   // subgrids may outlive the context
     if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     cudaFree(ctx->d_box);
     cudaFree(ctx->d_count);

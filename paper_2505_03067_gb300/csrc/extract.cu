@@ -537,6 +537,7 @@ mpm_status mpm_extract_impl(mpm_ctx *ctx, const mpm_lattice *lat, int32_t nspeci
     }
     for (int d = 0; d < 3; ++d) tmp.ldims[d] = lat->dims[d];
     tmp.hm = sub->hm;   // allocating the buffers above may have given them up
+    tmp.hm_ctx = sub->hm_ctx;
     tmp.hm_stride = sub->hm_stride;
     tmp.hm_cap = sub->hm_cap;
     tmp.hm_refused = sub->hm_refused;

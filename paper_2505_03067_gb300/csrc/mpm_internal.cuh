@@ -520,6 +520,7 @@ struct mpm_subgrid {
     // assembly and read by the solver; optional (mpm_face_means): without it the
     // solver forms them in every pass
     double *hm = nullptr;
+    mpm_ctx *hm_ctx = nullptr;           // the context whose hm_subs lists this subgrid (null: none)
     int64_t hm_stride = 0, hm_cap = 0;   // doubles per face, doubles allocated
     int64_t hm_refused = 0;              // doubles the device had no room for (0: not so far)
     bool hm_recorded = false;            // a caller's graph may hold its address (mpm_face_means_record)
@@ -544,7 +545,7 @@ mpm_status mpm_cuda_check(mpm_ctx *ctx, cudaError_t e, const char *what);
 cudaError_t mpm_dev_malloc(mpm_ctx *ctx, void **q, size_t bytes);
 mpm_status mpm_grow(mpm_ctx *ctx, void **p, size_t *cap, size_t need, const char *what);
 void mpm_face_means(mpm_ctx *ctx, mpm_subgrid *sub, int64_t n, int64_t room);   // a place for the face means of n elements, if any
-void mpm_face_means_free(mpm_ctx *ctx, mpm_subgrid *sub);
+void mpm_face_means_free(mpm_subgrid *sub);
 void mpm_face_means_record(mpm_subgrid *sub, cudaStream_t st);
 
 #define MPM_CU(call)                                                       \

@@ -187,3 +187,27 @@ def test_means_that_a_recorded_graph_writes_stay(M, case):
     uniform = M.DeviceLattice(W.random_case(31, (21, 13, 11), nspecies=3).lattice)
     sub.mpm_box_extract(uniform, 3, wl.margin)         # leaves the buffer to the graph
     assert held(M, ctx) == 0
+
+
+def test_a_subgrid_destroyed_without_its_context_leaves_nothing_behind(M, case):
+    """mpm_subgrid_destroy(NULL, sub) is allowed, before the context is destroyed
+    and after it."""
+    wl, states = case
+    ctx = M.Context(0)
+    a, b = System(M, ctx, wl, "step"), System(M, ctx, wl, "step")
+    a.step()
+    b.step()
+    one = held(M, ctx) // 2
+    h, a.sub.h = a.sub.h, None                          # the binding's own destroy has nothing left to do
+    assert ctx.lib.mpm_subgrid_destroy(None, h) == M.OK
+    assert held(M, ctx) == one
+    ctx.debug_set(M.DEBUG_REFUSE_ALLOC, 1)
+    c = System(M, ctx, wl, "step")
+    c.step()
+    b.step()
+    assert b.error(states) <= BOUND and c.error(states) <= BOUND
+    handles = [s.sub.h for s in (b, c)]
+    b.sub.h = c.sub.h = None
+    lib = ctx.lib
+    ctx.close()
+    assert [lib.mpm_subgrid_destroy(None, h) for h in handles] == [M.OK, M.OK]
