@@ -350,12 +350,13 @@ mpm_status mpm_tune_tile(mpm_ctx *ctx, const mpm_lattice *lat, int32_t margin, i
 /*
  * Autotuner, restart length and solver kernel variant for a batch of
  * assembled subgrids: times a warm-up and a measured solve from c^n for every
- * candidate (m in {4, 8, 16}; for FP32 with m <= 8 the 4 kernel variants) and
- * keeps the fastest that converges.  Writes m into opt->restart and the
+ * candidate (m in {4, 8, 16}; with m <= 8 the 7 kernel variants of FP32 or the
+ * 6 of FP64; variant 0 alone when a system of the batch has dfac, as such
+ * batches have no other) and keeps the fastest that converges.  Writes m into opt->restart and the
  * variant to *out_variant, and makes that variant the context's default.
  * cache_path (nullable) is a text file of earlier results, keyed by the GPU,
- * precision, tolerance and every system's bucketed box shape and mask
- * occupancy; a hit skips the timing, a miss appends a line.  The iterates are
+ * precision, tolerance and every system's bucketed box shape, mask occupancy
+ * and presence of dfac; a hit skips the timing, a miss appends a line.  The iterates are
  * left at c^n.
  */
 mpm_status mpm_tune_solver(mpm_ctx *ctx, mpm_subgrid *const *subs, int32_t nsys, mpm_opts *opt,
@@ -556,8 +557,8 @@ mpm_status mpm_scatter(mpm_ctx *ctx, const mpm_subgrid *sub, const mpm_lattice *
  *                        went (read with the MPM_COUNTER_PHASE_* counters).
  *  MPM_DEBUG_SOLVER_VARIANT  solver kernel variant 0..6 (elements in flight per
  *                        thread, CTAs per SM, threads per CTA; 0 = default;
- *                        a bucket without the variant uses its default), for
- *                        tuning.
+ *                        a bucket without the variant uses its default, and so
+ *                        does a solve of which a system has dfac), for tuning.
  *  MPM_DEBUG_CNN_LAYER_TIMES 1: every later network application outside a
  *                        graph capture records CUDA events around each of its
  *                        six convolution launches (read with

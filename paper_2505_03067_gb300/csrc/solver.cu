@@ -98,10 +98,11 @@ int mpm_solver_max_blocks(mpm_ctx *ctx, int prec, int m, int variant, bool var)
     return variant_max_blocks(ctx, pick(prec, maxm, variant, var), false);
 }
 
-// Number of kernel variants of a (precision, restart) bucket (for the tuner).
-int mpm_solver_variants(int prec, int m)
+// Number of kernel variants of a (precision, restart) bucket (for the tuner);
+// with a per-voxel diffusivity (var) pick knows only the default.
+int mpm_solver_variants(int prec, int m, bool var)
 {
-    if (m > 8) return 1;
+    if (m > 8 || var) return 1;
     return prec == 1 ? 7 : 6;
 }
 

@@ -10,7 +10,8 @@
 // timed with CUDA events; the fastest wins.  Results go to an optional
 // on-disk cache, one line per key: the GPU name, precision, tolerance, and
 // for every system its species count with bucketed box dims
-// (nearest power of two) and mask occupancy (tenths).
+// (nearest power of two), mask occupancy (tenths) and whether its diffusivity
+// varies (such batches run kernels of their own).
 #include <algorithm>
 #include <cmath>
 #include <cstdio>
@@ -20,7 +21,7 @@
 
 #include "mpm_internal.cuh"
 
-int mpm_solver_variants(int prec, int m);
+int mpm_solver_variants(int prec, int m, bool var);
 
 namespace {
 
@@ -50,6 +51,7 @@ std::string cache_key(mpm_ctx *ctx, mpm_subgrid *const *subs, int nsys, const mp
         snprintf(buf, sizeof(buf), ";%d:%d,%d,%d,%d", s->nspecies, ilog2(std::max(1, s->n[0])),
                  ilog2(std::max(1, s->n[1])), ilog2(std::max(1, s->n[2])), occ);
         k += buf;
+        if (s->has_dfac) k += ",D";
     }
     return k;
 }
@@ -142,8 +144,10 @@ extern "C" mpm_status mpm_tune_solver(mpm_ctx *ctx, mpm_subgrid *const *subs, in
     const int saved_var = ctx->solver_variant;
     double best_ms = 1e300;
     int best_m = opt->restart, best_v = 0;
+    bool any_var = false;
+    for (int i = 0; i < nsys; ++i) any_var |= subs[i]->has_dfac;
     for (int32_t mm : kRestarts) {
-        const int nvar = mpm_solver_variants(opt->precision, mm);
+        const int nvar = mpm_solver_variants(opt->precision, mm, any_var);
         for (int v = 0; v < nvar; ++v) {
             mpm_opts o = *opt;
             o.restart = mm;
