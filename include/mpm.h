@@ -587,6 +587,13 @@ mpm_status mpm_debug_set(mpm_ctx *ctx, int32_t key, int64_t value);
 mpm_status mpm_debug_convert(const double *in64, float *out32, float *ref32, const float *in32, double *out64,
                              double *ref64, int64_t n, void *stream);
 
+/* Test hook: the network's activation applied to n device values, GELU(z) =
+ * z Phi(z) in FP32 before it is rounded to bf16: out[i] as inference evaluates
+ * it, out_train[i] as a training step does.  Both give NaN at -infinity.  Device
+ * arrays of n entries; queued on `stream`.  MPM_ERR_ARG for n < 0 or a null
+ * pointer. */
+mpm_status mpm_debug_gelu(const float *z, float *out, float *out_train, int64_t n, void *stream);
+
 /* Counters of the context: MPM_COUNTER_LAUNCHES = kernels launched so far by
  * this context (every entry point counts its own launches); with
  * MPM_DEBUG_PHASE_TIMES on, the last solve's CTA-0 nanoseconds spent in the

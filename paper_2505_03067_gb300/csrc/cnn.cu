@@ -161,6 +161,15 @@ __global__ void k_adam(float *__restrict__ p, const float *__restrict__ g, float
     }
 }
 
+// The two forms of the activation, elementwise (test hook: mpm_debug_gelu).
+__global__ void k_debug_gelu(const float *__restrict__ z, float *__restrict__ out, float *__restrict__ out_train, int64_t n)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+        out[i] = tc::gelu(z[i]);
+        out_train[i] = tc::gelu_train(z[i]);
+    }
+}
+
 // ---------------------------------------------------------------- plans
 // Candidate unit ci of image mode -> unit record; false if it lies outside its image's box.
 __device__ __forceinline__ bool unit_of(const CnnDom &D, uint32_t ci, Unit &u)
@@ -1052,6 +1061,14 @@ extern "C" mpm_status mpm_cnn_layer_times(mpm_ctx *ctx, mpm_cnn *c, float ms[6])
     MPM_CU(cudaEventSynchronize(c->lev[kLayers]));
     for (int l = 0; l < kLayers; ++l) MPM_CU(cudaEventElapsedTime(&ms[l], c->lev[l], c->lev[l + 1]));
     return MPM_OK;
+}
+
+extern "C" mpm_status mpm_debug_gelu(const float *z, float *out, float *out_train, int64_t n, void *stream)
+{
+    if (n < 0 || (n > 0 && (!z || !out || !out_train))) return MPM_ERR_ARG;
+    if (n == 0) return MPM_OK;
+    k_debug_gelu<<<(int)std::min<int64_t>((n + 255) / 256, 4096), 256, 0, (cudaStream_t)stream>>>(z, out, out_train, n);
+    return cudaGetLastError() == cudaSuccess ? MPM_OK : MPM_ERR_CUDA;
 }
 
 extern "C" mpm_status mpm_cnn_destroy(mpm_ctx *ctx, mpm_cnn *c)

@@ -34,7 +34,7 @@ SYMBOLS = ["mpm_create", "mpm_destroy", "mpm_last_error", "mpm_subgrid_create", 
            "mpm_tune_tile", "mpm_tune_solver", "mpm_tune_teams", "mpm_cnn_create", "mpm_cnn_destroy", "mpm_cnn_set_params",
            "mpm_cnn_get_params", "mpm_cnn_load_image", "mpm_cnn_export_features", "mpm_cnn_export_preact", "mpm_cnn_forward", "mpm_cnn_train_step", "mpm_cnn_guess", "mpm_cnn_layer_times",
            "mpm_step", "mpm_step_enqueue", "mpm_step_wait", "mpm_solve_fgmres_cnn", "mpm_cnn_precond",
-           "mpm_step_host", "mpm_debug_convert", "mpm_step_set_network", "mpm_cpm_step"]
+           "mpm_step_host", "mpm_debug_convert", "mpm_debug_gelu", "mpm_step_set_network", "mpm_cpm_step"]
 
 
 class mpm_box(C.Structure):
@@ -160,6 +160,7 @@ def load(path: str = LIB_PATH) -> C.CDLL:
         "mpm_counter_get": [P, C.c_int32, C.POINTER(C.c_int64)],
         "mpm_box_bounds_noalloc": [P, C.POINTER(C.c_int32), C.c_int32, P, P],
         "mpm_debug_convert": [P, P, P, P, P, P, C.c_int64, P],
+        "mpm_debug_gelu": [P, P, P, C.c_int64, P],
         "mpm_cpm_step": [P, C.POINTER(mpm_lattice), C.POINTER(mpm_params), C.POINTER(mpm_cpm_params), C.c_uint64,
                          C.c_int64, P, P, P],
         "mpm_step_set_network": [P, P, P],
@@ -524,6 +525,20 @@ def mpm_debug_convert(in64, in32, stream=None):
     if st != OK:
         raise MpmError(st, "mpm_debug_convert failed")
     return out32, ref32, out64, ref64
+
+
+def mpm_debug_gelu(z, stream=None):
+    """The network's activation on a device tensor (test hook): returns it as
+    inference and as a training step evaluate it."""
+    import torch
+    if not (z.is_cuda and z.dtype == torch.float32 and z.is_contiguous()):
+        raise ValueError("mpm_debug_gelu: a contiguous CUDA float32 tensor")
+    out, out_train = torch.empty_like(z), torch.empty_like(z)
+    ptr = lambda t: C.c_void_p(t.data_ptr())  # noqa: E731
+    st = load().mpm_debug_gelu(ptr(z), ptr(out), ptr(out_train), z.numel(), _stream_ptr(stream))
+    if st != OK:
+        raise MpmError(st, "mpm_debug_gelu failed")
+    return out, out_train
 
 
 def mpm_solve_batch(ctx: Context, subs, opts: mpm_opts, scatter_to=None, stream=None, allow=(ERR_NOCONV,)):
