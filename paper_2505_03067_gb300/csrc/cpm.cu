@@ -429,10 +429,13 @@ extern "C" mpm_status mpm_cpm_step(mpm_ctx *ctx, const mpm_lattice *lat, const m
     cudaStream_t st = (cudaStream_t)stream;
     const int cap = prm->ncell;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    // a front voxel has a tumour neighbour, and a tumour voxel at most six of them: at most 6 L / 7
-    const size_t b_bits = al((size_t)((L + 31) / 32) * 4), b_front = al((size_t)(L - L / 7) * 4), b_vol = al((size_t)cap * 8), b_sum = al((size_t)cap * 24),
+    // a front voxel has a tumour neighbour, and a tumour voxel at most six of them: at most 6 L / 7.
+    // Bits, front and its count lie without padding between them: for every L they
+    // take no more than 4 L bytes rounded up to 256, which small contexts are made for.
+    const size_t nwords = (size_t)((L + 31) / 32), nfront = (size_t)(L - L / 7);
+    const size_t b_lat = al((2 * nwords + nfront + 1) * 4), b_vol = al((size_t)cap * 8), b_sum = al((size_t)cap * 24),
                  b_i = al((size_t)(cap + 1) * 4);
-    mpm_status r = mpm_grow(ctx, (void **)&ctx->d_cpm, &ctx->cpm_cap, 2 * b_bits + b_front + 256 + b_vol + b_sum + 2 * b_i,
+    mpm_status r = mpm_grow(ctx, (void **)&ctx->d_cpm, &ctx->cpm_cap, b_lat + b_vol + b_sum + 2 * b_i,
                             "growth driver scratch");
     if (r != MPM_OK) return r;
     char *p = (char *)ctx->d_cpm;
@@ -440,12 +443,11 @@ extern "C" mpm_status mpm_cpm_step(mpm_ctx *ctx, const mpm_lattice *lat, const m
     memset(&A, 0, sizeof(A));
     A.cell = const_cast<int32_t *>(lat->cell_id);   // updated in place (documented)
     A.bits = (uint32_t *)p;
-    A.grown = (uint32_t *)(p + b_bits);
-    A.nwords = (uint32_t)((L + 31) / 32);
-    A.front = (uint32_t *)(p + 2 * b_bits);
-    p += 2 * b_bits + b_front;
-    A.nfront = (uint32_t *)p;
-    p += 256;
+    A.grown = A.bits + nwords;
+    A.nwords = (uint32_t)nwords;
+    A.front = A.grown + nwords;
+    p += b_lat;
+    A.nfront = (uint32_t *)p - 1;   // just before the sums: zeroed with them
     A.vol = (unsigned long long *)p;
     A.sum = (unsigned long long *)(p + b_vol);
     A.daughter = (int32_t *)(p + b_vol + b_sum);
@@ -470,7 +472,7 @@ extern "C" mpm_status mpm_cpm_step(mpm_ctx *ctx, const mpm_lattice *lat, const m
     A.stats = (unsigned long long *)stats_dev;
     A.seed = seed;
     A.step = step;
-    MPM_CU(cudaMemsetAsync(A.nfront, 0, 256 + b_vol + b_sum, st));
+    MPM_CU(cudaMemsetAsync(A.nfront, 0, sizeof(uint32_t) + b_vol + b_sum, st));
     k_cpm_scan<<<ctx->num_sms * 6, 256, 0, st>>>(A);
     k_cpm_front<<<(A.nwords + kGrowWords - 1) / kGrowWords, kGrowWords, 0, st>>>(A);
     k_cpm_grow<<<ctx->num_sms * 4, 256, 0, st>>>(A);
