@@ -266,7 +266,6 @@ struct Halo {
     static constexpr int QP = QC + (QC & 1);
     static constexpr int GS = QP * 128;            // bytes per halo row (18 of them per depth)
     static constexpr int SLOT = kHaloY * GS;       // bytes per depth
-    static constexpr int NKS = QP / 2;             // MMAs of K = 16 per tap
 };
 
 // The forward kernel's staged halo depth: the voxels once, [halo row y'][chunk
