@@ -3,7 +3,7 @@
 // Sec. 2.1 / 2.4; the paper gives no Hamiltonian, so this is one simple
 // rule, stated in the C header).
 //
-// Five launches per step, all stream-ordered, no host round trip.  The lattice
+// Five launches per step (four on a small lattice), all stream-ordered, no host round trip.  The lattice
 // is read once: one bit per voxel (tumour or not) stands in for it afterwards,
 // so that only the words of the tumour and of its front are touched again.
 //   k_cpm_scan     lattice -> tumour bits; per-cell volume and coordinate sums
@@ -26,6 +26,12 @@
 // with a full-lattice pass per launch (grow 495, stats 196, plan 28, apply
 // 149 us) and takes 152 us now (scan 63, front 27, grow 9, plan 13, apply 3, or
 // 21 us when cells divide), against 56 us for one reading of ids and mask.
+// Small lattices (kSmallWords) are a chain of short launches, each as long as
+// its slowest warp's loads: there the scan gives a warp one word at a time, and
+// the front kernel takes 32 words a CTA and decides the growth itself.  A step
+// on 64^3 takes 28 us so and 32 us in the other form (27 us with a full-lattice
+// pass per launch), on 128^3 29 against 33, on 192^3 48 against 41; around 160^3
+// it depends on the tumour's surface (37 against 39, 42 against 39.5).
 // Randomness: SplitMix64's output function on a counter (seed, step, stream,
 // index), so the decisions do not depend on the launch shape.
 #include <cmath>
@@ -50,6 +56,8 @@ __device__ __forceinline__ uint64_t cpm_draw(uint64_t seed, int64_t step, int st
     const uint64_t c = ((uint64_t)((4 * step + stream) & ((1 << 24) - 1)) << 40) | idx;
     return splitmix_out(seed + (c + 1ull) * kGamma);
 }
+
+constexpr uint32_t kSmallWords = 1u << 16;   // 2 M voxels: the line between the two forms
 
 struct CpmArgs {
     int32_t *cell;               // lattice cell ids (in: before the step, out: after)
@@ -109,12 +117,12 @@ __device__ __forceinline__ void cpm_count_row(const CpmArgs &A, unsigned lanes, 
 }
 
 // Bound by HBM: 4 bytes read and an eighth of a byte written per voxel.  A warp
-// takes kScanWords consecutive words at a time, loads the next ones (coalesced
+// takes kScanWords (8; small lattices 1) consecutive words at a time, loads the next ones (coalesced
 // 128-byte loads) before it works on these, keeps word k in lane k and stores
 // them together; a word without any id is done after its vote.  63 us on the
 // 512x384x384 lattice (4.8 TB/s); 81 us with 16 words a warp, no load ahead and
 // the sums by warp reductions.
-constexpr int kScanWords = 8;
+template <int kScanWords>
 __global__ void __launch_bounds__(256, 6) k_cpm_scan(const __grid_constant__ CpmArgs A)
 {
     const int lane = threadIdx.x & 31;
@@ -172,25 +180,70 @@ __device__ __forceinline__ uint32_t cpm_bits(const CpmArgs &A, int64_t p)
 
 __device__ __forceinline__ bool cpm_tumour(const CpmArgs &A, uint32_t v) { return (A.bits[v >> 5] >> (v & 31)) & 1u; }
 
+// The growth of front voxel v: the id that takes it over (written), or 0.
+__device__ __forceinline__ int32_t cpm_take(const CpmArgs &A, uint32_t v)
+{
+    const uint32_t Lx = A.Lx, Ly = A.Ly, Lz = A.Lz, Lxy = Lx * Ly;
+    const double c0 = A.o2[v], c1 = A.nut[v];
+    const uint32_t row = v / Lx, x = v - row * Lx, z = row / Ly, y = row - z * Ly;
+    uint32_t tm = 0;   // tumour neighbours -x, +x, -y, +y, -z, +z
+    if (x > 0 && cpm_tumour(A, v - 1)) tm |= 1u;
+    if (x + 1 < Lx && cpm_tumour(A, v + 1)) tm |= 2u;
+    if (y > 0 && cpm_tumour(A, v - Lx)) tm |= 4u;
+    if (y + 1 < Ly && cpm_tumour(A, v + Lx)) tm |= 8u;
+    if (z > 0 && cpm_tumour(A, v - Lxy)) tm |= 16u;
+    if (z + 1 < Lz && cpm_tumour(A, v + Lxy)) tm |= 32u;
+    if (!tm || c0 < A.o2_min) return 0;
+    // same operations, same order as the rule's statement (no contraction possible)
+    const double p = A.p_grow * (c0 / (A.K_o2 + c0)) * (c1 / (A.K_nut + c1));
+    const double u = (double)(cpm_draw(A.seed, A.step, 0, (uint64_t)v) >> 11) * 0x1.0p-53;
+    if (!(u < p)) return 0;
+    const uint64_t h = cpm_draw(A.seed, A.step, 1, (uint64_t)v) >> 32;
+    const uint32_t j = (uint32_t)((h * (uint32_t)__popc(tm)) >> 32);
+    uint32_t t = tm;   // the j-th tumour neighbour
+    for (uint32_t r = 0; r < j; ++r) t &= t - 1;
+    const uint32_t d = __ffs(t) - 1;
+    const uint32_t o = d < 2 ? 1u : d < 4 ? Lx : Lxy;
+    const int32_t out = A.cell[(d & 1) ? v + o : v - o];
+    A.cell[v] = out;
+    atomicOr(A.grown + (v >> 5), 1u << (v & 31));
+    return out;
+}
+
+// Counts a warp's growth (out: what cpm_take gave, 0 at lanes without a voxel).
+__device__ __forceinline__ void cpm_count_growth(const CpmArgs &A, int32_t out, uint32_t v)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned g = __ballot_sync(0xffffffffu, out > 0);
+    const unsigned okm = __ballot_sync(0xffffffffu, out > 0 && out < A.cap);
+    if (lane == 0 && g) {
+        atomicAdd(A.stats + 0, (unsigned long long)__popc(g));
+        if (g != okm) atomicAdd(A.stats + 2, (unsigned long long)__popc(g & ~okm));
+    }
+    if ((okm >> lane) & 1u) cpm_count(A, okm, out, v);
+}
+
 // The medium voxels of the mask next to a tumour voxel, to a list.  A CTA takes
-// 256 words (8192 voxels): a thread dilates one word of the bits (six shifted
+// kWords (256: 8192 voxels; small lattices 32) words: a thread dilates one word of the bits (six shifted
 // words, all in L2), the voxels of the dilation that are no tumour go to a list
 // in shared memory, and the CTA's threads look at the mask and the id of the
 // list's voxels.  The dilation ignores the lattice's faces; k_cpm_grow looks at
-// them.  Bound by latency, hence the small kernel with eight CTAs on an SM;
-// deciding the growth here as well (two FP64 divisions a voxel, few lanes of a
-// warp) took 51 us against 27 + 9 us on the 512x384x384 lattice.
-constexpr int kGrowWords = 256;
-__global__ void __launch_bounds__(kGrowWords, 8) k_cpm_front(const __grid_constant__ CpmArgs A)
+// them.  Bound by latency, hence the small kernel with eight CTAs on an SM.
+// kGrow: the growth is decided here as well, without the list.  That saves a
+// launch; on the 512x384x384 lattice (two FP64 divisions a voxel, few lanes of a
+// warp) it took 51 us against 27 + 9 us.
+constexpr int kFrontThreads = 256;
+template <int kWords, bool kGrow>
+__global__ void __launch_bounds__(kFrontThreads, 8) k_cpm_front(const __grid_constant__ CpmArgs A)
 {
-    __shared__ uint16_t s_list[kGrowWords * 32];
+    __shared__ uint16_t s_list[kWords * 32];
     __shared__ int s_n;
     const uint32_t Lx = A.Lx, Lxy = Lx * (uint32_t)A.Ly;
-    const uint32_t w = blockIdx.x * kGrowWords + threadIdx.x;
+    const uint32_t w = blockIdx.x * kWords + threadIdx.x;
     const int64_t v0 = (int64_t)w * 32;
     uint32_t cand = 0u;
     if (threadIdx.x == 0) s_n = 0;
-    if (w < A.nwords) {
+    if (threadIdx.x < kWords && w < A.nwords) {
         const uint32_t own = A.bits[w];
         cand = (cpm_bits(A, v0 - 1) | cpm_bits(A, v0 + 1) | cpm_bits(A, v0 - Lx) | cpm_bits(A, v0 + Lx) |
                 cpm_bits(A, v0 - Lxy) | cpm_bits(A, v0 + Lxy)) & ~own;
@@ -204,10 +257,14 @@ __global__ void __launch_bounds__(kGrowWords, 8) k_cpm_front(const __grid_consta
     }
     __syncthreads();
     const int n = s_n, lane = threadIdx.x & 31;
-    for (int i0 = threadIdx.x & ~31; i0 < n; i0 += kGrowWords) {   // warp-uniform: the vote is legal inside
+    for (int i0 = threadIdx.x & ~31; i0 < n; i0 += kFrontThreads) {   // warp-uniform: the vote is legal inside
         const int i = i0 + lane;
-        const uint32_t v = blockIdx.x * (kGrowWords * 32u) + (i < n ? s_list[i] : 0);
+        const uint32_t v = blockIdx.x * (kWords * 32u) + (i < n ? s_list[i] : 0);
         const bool front = i < n && A.mask[v] != 0 && A.cell[v] == 0;
+        if (kGrow) {
+            cpm_count_growth(A, front ? cpm_take(A, v) : 0, v);
+            continue;
+        }
         const unsigned f = __ballot_sync(0xffffffffu, front);
         if (!f) continue;
         uint32_t at = 0;
@@ -220,49 +277,12 @@ __global__ void __launch_bounds__(kGrowWords, 8) k_cpm_front(const __grid_consta
 // The growth of the listed voxels, spread evenly over the GPU.
 __global__ void __launch_bounds__(256) k_cpm_grow(const __grid_constant__ CpmArgs A)
 {
-    const uint32_t Lx = A.Lx, Ly = A.Ly, Lz = A.Lz, Lxy = Lx * Ly;
     const uint32_t n = *A.nfront, lane = threadIdx.x & 31;
     for (uint32_t i0 = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n; i0 += gridDim.x * blockDim.x) {
-        int32_t out = 0;
-        uint32_t v = 0;
-        if (i0 + lane < n) {
-            v = A.front[i0 + lane];
-            const double c0 = A.o2[v], c1 = A.nut[v];
-            const uint32_t row = v / Lx, x = v - row * Lx, z = row / Ly, y = row - z * Ly;
-            uint32_t tm = 0;   // tumour neighbours -x, +x, -y, +y, -z, +z
-            if (x > 0 && cpm_tumour(A, v - 1)) tm |= 1u;
-            if (x + 1 < Lx && cpm_tumour(A, v + 1)) tm |= 2u;
-            if (y > 0 && cpm_tumour(A, v - Lx)) tm |= 4u;
-            if (y + 1 < Ly && cpm_tumour(A, v + Lx)) tm |= 8u;
-            if (z > 0 && cpm_tumour(A, v - Lxy)) tm |= 16u;
-            if (z + 1 < Lz && cpm_tumour(A, v + Lxy)) tm |= 32u;
-            if (tm && !(c0 < A.o2_min)) {
-                // same operations, same order as the rule's statement (no contraction possible)
-                const double p = A.p_grow * (c0 / (A.K_o2 + c0)) * (c1 / (A.K_nut + c1));
-                const double u = (double)(cpm_draw(A.seed, A.step, 0, (uint64_t)v) >> 11) * 0x1.0p-53;
-                if (u < p) {
-                    const uint64_t h = cpm_draw(A.seed, A.step, 1, (uint64_t)v) >> 32;
-                    const uint32_t j = (uint32_t)((h * (uint32_t)__popc(tm)) >> 32);
-                    uint32_t t = tm;   // the j-th tumour neighbour
-                    for (uint32_t r = 0; r < j; ++r) t &= t - 1;
-                    const uint32_t d = __ffs(t) - 1;
-                    const uint32_t o = d < 2 ? 1u : d < 4 ? Lx : Lxy;
-                    out = A.cell[(d & 1) ? v + o : v - o];
-                    A.cell[v] = out;
-                    atomicOr(A.grown + (v >> 5), 1u << (v & 31));
-                }
-            }
-        }
-        const unsigned g = __ballot_sync(0xffffffffu, out > 0);
-        const unsigned okm = __ballot_sync(0xffffffffu, out > 0 && out < A.cap);
-        if (lane == 0 && g) {
-            atomicAdd(A.stats + 0, (unsigned long long)__popc(g));
-            if (g != okm) atomicAdd(A.stats + 2, (unsigned long long)__popc(g & ~okm));
-        }
-        if ((okm >> lane) & 1u) cpm_count(A, okm, out, v);
+        const uint32_t v = i0 + lane < n ? A.front[i0 + lane] : 0u;
+        cpm_count_growth(A, i0 + lane < n ? cpm_take(A, v) : 0, v);
     }
 }
-
 // One CTA: daughters in increasing parent id order while the tables have room.
 // Bound by the latency of its loads: a round takes kPlanRun ids per thread (ids
 // 1024 apart, so that all accesses are coalesced, with all volumes in flight),
@@ -430,10 +450,12 @@ extern "C" mpm_status mpm_cpm_step(mpm_ctx *ctx, const mpm_lattice *lat, const m
     const int cap = prm->ncell;
     auto al = [](size_t b) { return (b + 255) & ~(size_t)255; };
     // a front voxel has a tumour neighbour, and a tumour voxel at most six of them: at most 6 L / 7.
-    // Bits, front and its count lie without padding between them: for every L they
-    // take no more than 4 L bytes rounded up to 256, which small contexts are made for.
+    // Bits, front and its count lie close together (the bits on 128-byte boundaries
+    // where there is room): for every L they take no more than 4 L bytes rounded up
+    // to 256, which small contexts are made for.
     const size_t nwords = (size_t)((L + 31) / 32), nfront = (size_t)(L - L / 7);
-    const size_t b_lat = al((2 * nwords + nfront + 1) * 4), b_vol = al((size_t)cap * 8), b_sum = al((size_t)cap * 24),
+    const size_t bits = L < 4096 ? nwords : (nwords + 31) & ~(size_t)31;
+    const size_t b_lat = al((2 * bits + nfront + 1) * 4), b_vol = al((size_t)cap * 8), b_sum = al((size_t)cap * 24),
                  b_i = al((size_t)(cap + 1) * 4);
     mpm_status r = mpm_grow(ctx, (void **)&ctx->d_cpm, &ctx->cpm_cap, b_lat + b_vol + b_sum + 2 * b_i,
                             "growth driver scratch");
@@ -443,9 +465,9 @@ extern "C" mpm_status mpm_cpm_step(mpm_ctx *ctx, const mpm_lattice *lat, const m
     memset(&A, 0, sizeof(A));
     A.cell = const_cast<int32_t *>(lat->cell_id);   // updated in place (documented)
     A.bits = (uint32_t *)p;
-    A.grown = A.bits + nwords;
+    A.grown = A.bits + bits;
     A.nwords = (uint32_t)nwords;
-    A.front = A.grown + nwords;
+    A.front = A.grown + bits;
     p += b_lat;
     A.nfront = (uint32_t *)p - 1;   // just before the sums: zeroed with them
     A.vol = (unsigned long long *)p;
@@ -474,11 +496,17 @@ extern "C" mpm_status mpm_cpm_step(mpm_ctx *ctx, const mpm_lattice *lat, const m
     A.step = step;
     // from a 256-byte boundary on (an unaligned fill cost 1 us): what lies there before the count is written later
     MPM_CU(cudaMemsetAsync(p - 256, 0, 256 + b_vol + b_sum, st));
-    k_cpm_scan<<<ctx->num_sms * 6, 256, 0, st>>>(A);
-    k_cpm_front<<<(A.nwords + kGrowWords - 1) / kGrowWords, kGrowWords, 0, st>>>(A);
-    k_cpm_grow<<<ctx->num_sms * 4, 256, 0, st>>>(A);
+    const bool small = A.nwords <= kSmallWords;
+    if (small) {
+        k_cpm_scan<1><<<ctx->num_sms * 6, 256, 0, st>>>(A);
+        k_cpm_front<32, true><<<(A.nwords + 31) / 32, kFrontThreads, 0, st>>>(A);
+    } else {
+        k_cpm_scan<8><<<ctx->num_sms * 6, 256, 0, st>>>(A);
+        k_cpm_front<256, false><<<(A.nwords + 255) / 256, kFrontThreads, 0, st>>>(A);
+        k_cpm_grow<<<ctx->num_sms * 4, 256, 0, st>>>(A);
+    }
     k_cpm_plan<<<1, kPlanThreads, 0, st>>>(A);
     k_cpm_apply<<<ctx->num_sms * 8, 256, 0, st>>>(A);
-    ctx->launches += 5;
+    ctx->launches += small ? 4 : 5;
     return mpm_cuda_check(ctx, cudaGetLastError(), "cpm_step");
 }
