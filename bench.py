@@ -54,6 +54,14 @@ def _peaks():
         return 6800.0, "fallback"
 
 
+def _bf16_peak():
+    p = os.path.join(ROOT, "MEASURED_PEAKS.json")
+    try:
+        return float(json.load(open(p))["bf16_tflops"]), "measured"
+    except Exception:
+        return 1900.0, "fallback"
+
+
 def solver_bytes(rep, NM, NE, bT):
     """Algorithmic bytes of one solver launch: per in-mask voxel (the unknowns,
     NM) and species, R = x, b, diag64 (8 each) + write u0 (bT);
@@ -516,12 +524,13 @@ def cnn_layer_roofline(mpm, ctx, cnn, solver, stream, flush, active, reps=5):
     hid = float(np.mean(med[1:5]))
     flops = active * 27 * 24 * 24 * 2
     achieved = flops / (hid / 1e3) / 1e12
+    peak, src = _bf16_peak()
     rec = _traffic_record_cnn()
     traffic = rec["dram_bytes_per_launch"] * active / rec["active_voxels"] if rec else None
     return {"bound": "tensor", "kernel": "k_conv_tc<24, 32, 0> (hidden-layer 3x3x3 convolution, tcgen05)",
-            "achieved": achieved, "peak": 1980.0, "unit": "TFLOP/s", "frac": achieved / 1980.0,
+            "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
             "traffic": traffic, "flops_per_launch": flops, "ms_per_launch": hid, "layer_ms": med,
-            "peak_source": "measured bf16 burst (MEASURED_PEAKS.json bf16_tflops)",
+            "peak_source": f"{src} bf16 burst (MEASURED_PEAKS.json bf16_tflops)",
             "traffic_source": ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the same kernel on the "
                                "growth crop's largest state, scaled by active voxels (profiles/conv_tc_traffic.json)"
                                if rec else "no record for the current kernel sources")}
@@ -822,10 +831,10 @@ def main():
             r["roofline_cnn"] = {"bound": "tensor", "kernel": "the network's guess on the last sampled state: plan, "
                                  "features and six tcgen05 convolutions (k_conv_tc)",
                                  "achieved": last_mask * CNN_FLOPS_PER_VOXEL / t_cnn / 1e12,
-                                 "peak": 1980.0, "unit": "TFLOP/s", "peak_source": "measured bf16 burst "
-                                 "(MEASURED_PEAKS.json bf16_tflops)",
+                                 "peak": _bf16_peak()[0], "unit": "TFLOP/s",
+                                 "peak_source": f"{_bf16_peak()[1]} bf16 burst (MEASURED_PEAKS.json bf16_tflops)",
                                  "flops_per_launch": last_mask * CNN_FLOPS_PER_VOXEL, "ms": r["cnn_ms_last_step"]}
-            r["roofline_cnn"]["frac"] = r["roofline_cnn"]["achieved"] / 1980.0
+            r["roofline_cnn"]["frac"] = r["roofline_cnn"]["achieved"] / r["roofline_cnn"]["peak"]
         r["roofline_hbm"] = {"bound": "hbm", "achieved": r["kernel_bytes"] / sec / 1e9, "peak": peak, "unit": "GB/s",
                              "frac": r["kernel_bytes"] / sec / 1e9 / peak,
                              "peak_source": f"{src} (MEASURED_PEAKS.json hbm_gbs)",
