@@ -264,8 +264,10 @@ mpm_status mpm_batch_step(mpm_ctx *ctx, mpm_subgrid *const *subs, const mpm_latt
  * Device memory per subgrid: about (5 + 36 S) bytes per lattice voxel for the
  * element buffers plus (m + 1) S 4 (FP32 Krylov) or 8 (FP64) bytes per voxel
  * for the Krylov bases (S species, m the restart length), padded to tiles; with
- * dfac 8 more for its copy, and 48 more for its means across the faces (a
- * context with a memory cap, or a device without room, goes without them).
+ * dfac 8 more for its copy, and 48 more for its means across the faces.  The
+ * means only save time: a context with a memory cap, or a device without room,
+ * goes without them, and they are given up when another allocation of the
+ * context finds no room (unless a CUDA graph of the caller's recorded them).
  */
 mpm_status mpm_step(mpm_ctx *ctx, mpm_subgrid *sub, const mpm_lattice *lat, const mpm_params *prm, int32_t margin,
                     const int32_t tile[3], const mpm_opts *opt, mpm_report *rep, mpm_box *out_box, void *stream);

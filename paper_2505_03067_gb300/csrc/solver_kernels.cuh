@@ -269,7 +269,7 @@ __device__ __forceinline__ T open_sum_hm(const T *__restrict__ u, const double *
 // 48 bytes an element; the other form is for a subgrid without them.  On a
 // 97x150x121 lattice with four species in FP64 (193 k unknowns) extraction,
 // assembly, solve and scatter took 1570 us with the means formed in every pass
-// (solve 1175, assembly 193) and take 632 us with stored ones.
+// (solve 1175, assembly 193) and take 620 us with stored ones.
 enum { D_UNIFORM = 0, D_MEANS = 1, D_STORED = 2 };
 
 // Every pass handles U elements per thread and iteration (e, e+es, ...,
