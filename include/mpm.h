@@ -354,12 +354,13 @@ mpm_status mpm_tune_tile(mpm_ctx *ctx, const mpm_lattice *lat, int32_t margin, i
  * assembled subgrids: times a warm-up and a measured solve from c^n for every
  * candidate (m in {4, 8, 16}; with m <= 8 the 7 kernel variants of FP32 or the
  * 6 of FP64; variant 0 alone when a system of the batch has dfac, as such
- * batches have no other) and keeps the fastest that converges.  Writes m into opt->restart and the
- * variant to *out_variant, and makes that variant the context's default.
+ * batches have no other) and keeps the fastest that converges.  Writes m into
+ * opt->restart and the variant to *out_variant, and makes that variant the
+ * context's default.
  * cache_path (nullable) is a text file of earlier results, keyed by the GPU,
  * precision, tolerance and every system's bucketed box shape, mask occupancy
- * and presence of dfac; a hit skips the timing, a miss appends a line.  The iterates are
- * left at c^n.
+ * and presence of dfac; a hit skips the timing, a miss appends a line.  The
+ * iterates are left at c^n.
  */
 mpm_status mpm_tune_solver(mpm_ctx *ctx, mpm_subgrid *const *subs, int32_t nsys, mpm_opts *opt,
                            int32_t *out_variant, const char *cache_path, void *stream);

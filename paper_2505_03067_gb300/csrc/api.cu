@@ -5,7 +5,6 @@
 #include <cstdio>
 #include <cstring>
 #include <new>
-#include <vector>
 
 #include "mpm_internal.cuh"
 
@@ -46,15 +45,15 @@ cudaError_t mpm_dev_malloc(mpm_ctx *ctx, void **q, size_t bytes)
 {
     const cudaError_t e = try_malloc(ctx, q, bytes);
     if (e != cudaErrorMemoryAllocation) return e;
-    std::vector<mpm_subgrid *> subs;
-    for (mpm_subgrid *sub : ctx->hm_subs)
-        if (!sub->hm_recorded) subs.push_back(sub);
-    if (subs.empty()) return e;
-    for (mpm_subgrid *sub : subs) {
+    bool any = false;
+    for (size_t i = ctx->hm_subs.size(); i-- > 0;) {   // each one given up leaves the list
+        mpm_subgrid *sub = ctx->hm_subs[i];
+        if (sub->hm_recorded) continue;
         sub->hm_refused = sub->hm_cap;
         mpm_face_means_free(sub);
+        any = true;
     }
-    return try_malloc(ctx, q, bytes);
+    return any ? try_malloc(ctx, q, bytes) : e;
 }
 
 // Grow-only device buffer under the context's cap; the old contents are not kept.
